@@ -124,6 +124,7 @@ static dmts_status load_model(dmts_ctx *ctx, const dmts_model *in, bool is_nc, D
     if (in->n_weights != expect || !in->weights)
         return fail(ctx, DMTS_E_INVALID, "weight blob size does not match the model sizes");
     std::vector<float> h(in->weights, in->weights + expect);
+    if (is_nc) h.resize(expect + (size_t)m.nl * S * K);   // room for UW
     if (!upload(m, h)) return fail(ctx, DMTS_E_OOM, "weight upload failed");
     m.n_weights = (size_t)expect;
     // offsets (same order as the blob)
@@ -145,6 +146,8 @@ static dmts_status load_model(dmts_ctx *ctx, const dmts_model *in, bool is_nc, D
         const int H = K + m.nl;
         m.U = take((size_t)m.nl * C);
         m.Wqk = take((size_t)2 * H * m.nc * C);   // Wq rows then Wk rows: one [2 H n_c][C] matrix
+        m.UW = take((size_t)m.nl * S * K);
+        launch_tensor_head_weights(C, S, m.nl, m.emb, m.wrad[0], m.U, m.UW, nullptr);
     }
     if (m.bf16) {
         // split-bf16 host copies, K-major: each output row of the logical
@@ -246,6 +249,18 @@ static Epi epi(int mode) {
     return e;
 }
 
+static FirstIO first_io(dmts_ctx *ctx, const SysView &s, const DevModel &m) {
+    FirstIO f;
+    memset(&f, 0, sizeof f);
+    f.species = s.species;
+    f.emb = m.emb;
+    f.wrad = m.wrad[0];
+    f.n_species = m.S;
+    f.nu = m.nu;
+    f.err = ctx->d_err;
+    return f;
+}
+
 // One node-level contraction: the tensor cores (split-bf16 operands) for a
 // model that runs its MLPs in bf16, whatever the number of rows M (a batch
 // smaller than one 128-row tile reads zero-filled rows), so that an atom's
@@ -307,9 +322,16 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
         io.q = q;
         io.q_bf16 = q_bf;
         io.err = ctx->d_err;
-        {
+        if (t == 0) {
+            FirstIO f = first_io(ctx, s, m);
+            f.A = io.A;
+            f.q = bf ? nullptr : q;             // the tensor-core path reads only the split-bf16 copy
+            f.q_bf16 = q_bf;
+            ProfScope ps(ctx, "first_fwd", st);
+            launch_first_fwd(C, m.lmax, g, f, st);
+        } else {
             ProfScope ps(ctx, "mp_fwd", st);
-            if (bf && mp_fwd_tc_supported(C, m.K, io)) launch_mp_fwd_tc(m.lmax, g, io, m.nseg, ctx->d_err, st);
+            if (bf && mp_fwd_tc_supported(C, m.K)) launch_mp_fwd_tc(m.lmax, g, io, m.nseg, ctx->d_err, st);
             else launch_mp_fwd(C, m.lmax, m.K, g, io, st);
         }
         Epi e1 = epi(EPI_BIAS_SILU);
@@ -353,6 +375,21 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
             ed.out_bf16 = act_bf;
             if (!contract(ctx, m, N, C, C, gin, gin_bf, m.w2[t], 0, m.w2t_bf[t], ed, st, "gemm_tc", "gemm"))
                 return DMTS_E_CUDA;
+            if (t == 0) {
+                // dU/dq in q's buffer; the first layer's adjoint forms gA itself
+                Epi ev = epi(EPI_STORE);
+                ev.out = q;
+                if (!contract(ctx, m, N, NL * C, C, act, act_bf, m.w1[t], 0, m.w1t_bf[t], ev, st, "gemm_tc", "gemm"))
+                    return DMTS_E_CUDA;
+                FirstIO f = first_io(ctx, s, m);
+                f.A = A;
+                f.gq = q;
+                f.Ffix = (unsigned long long *)w.cons_ffix.p;
+                f.Wfix = virial ? (unsigned long long *)w.cons_wfix.p : nullptr;
+                ProfScope ps(ctx, "first_bwd", st);
+                launch_first_bwd(C, m.lmax, g, f, st);
+                break;
+            }
             Epi ea = epi(EPI_GA);
             ea.A = A + nc_ * NLM * t;
             ea.out = gA;
@@ -367,8 +404,8 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
             io.nu = m.nu;
             io.gA = gA;
             io.gs_in = gin;
-            io.gs_out = t > 0 ? gout : nullptr;   // layer 0's inputs are the species embedding
-            io.gs_out_bf16 = t > 0 ? gout_bf : nullptr;
+            io.gs_out = gout;
+            io.gs_out_bf16 = gout_bf;
             io.Ffix = (unsigned long long *)w.cons_ffix.p;
             io.Wfix = virial ? (unsigned long long *)w.cons_wfix.p : nullptr;
             io.err = ctx->d_err;
@@ -440,19 +477,16 @@ dmts_status nc_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const i
     float *s0 = (float *)w.nc_s.p, *s1 = s0 + nc_;
     const EdgeGeom g = edge_geom(s, row_ptr, col, m);
     if (!(flags & kFlagEmbedded)) { ProfScope ps(ctx, "embed", st); launch_embed(N, C, s.species, m.emb, s0, st); }
-    LayerIO io;
-    memset(&io, 0, sizeof io);
-    io.s = s0;
-    io.wrad = m.wrad[0];
-    io.nu = m.nu;
+    FirstIO io = first_io(ctx, s, m);
     io.A = (flags & kFlagKeepPre) ? (float *)w.dist_A.p : nullptr;   // the head needs q and V only; kept for the distillation
-    io.q = (float *)w.nc_q.p;
+    // the tensor-core path reads only the split-bf16 copy; the distillation's
+    // weight gradient reads the fp32 one
+    io.q = (bf && !(flags & kFlagKeepPre)) ? nullptr : (float *)w.nc_q.p;
     io.q_bf16 = q_bf;
-    io.U = m.U;
+    io.UW = m.UW;
     io.V = (float *)w.nc_v.p;
     io.n_l = m.nl;
-    io.err = ctx->d_err;
-    { ProfScope ps(ctx, "nc_mp_fwd", st); launch_mp_fwd(C, 1, m.K, g, io, st); }
+    { ProfScope ps(ctx, "nc_mp_fwd", st); launch_first_fwd(C, 1, g, io, st); }
     Epi e1 = epi(EPI_BIAS_SILU);
     e1.bias = m.b1[0];
     e1.H = (flags & kFlagKeepPre) ? (float *)w.dist_h.p : nullptr;   // kept only for the distillation
@@ -460,7 +494,7 @@ dmts_status nc_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const i
     // weight gradient reads the fp32 activation
     e1.out = (bf && !(flags & kFlagKeepPre)) ? nullptr : (float *)w.nc_act.p;
     e1.out_bf16 = act_bf;
-    if (!contract(ctx, m, N, C, 2 * C, io.q, q_bf, m.w1[0], 1, m.w1_bf[0], e1, st, "nc_gemm_tc", "nc_gemm"))
+    if (!contract(ctx, m, N, C, 2 * C, (float *)w.nc_q.p, q_bf, m.w1[0], 1, m.w1_bf[0], e1, st, "nc_gemm_tc", "nc_gemm"))
         return DMTS_E_CUDA;
     Epi e2 = epi(EPI_RESID);
     e2.bias = m.b2[0];
@@ -1102,6 +1136,7 @@ dmts_status nc_distill_step(dmts_ctx *ctx, const dmts_system *sys, const dmts_nb
         if (fit_layer) {
             adam(m.wrad[0], (size_t)2 * m.K * C, nullptr, 1);
             adam(m.U, (size_t)m.nl * C, nullptr, 1);
+            launch_tensor_head_weights(C, m.S, m.nl, m.emb, m.wrad[0], m.U, m.UW, st);
         }
         if (fit_mlp) {
             adam(m.w1[0], (size_t)C * 2 * C, m.bf16 ? m.w1_bf[0] : nullptr, 2 * C);

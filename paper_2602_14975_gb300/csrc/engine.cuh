@@ -33,6 +33,7 @@ struct DevModel {
           *w2[DMTS_MAX_LAYERS] = {}, *b2[DMTS_MAX_LAYERS] = {};
     float *wr = nullptr, *br = nullptr, *wo = nullptr;
     float *U = nullptr, *Wqk = nullptr;
+    float *UW = nullptr;                  // [n_l][S][K] of the first layer (launch_tensor_head_weights), after the blob
     // split-bf16 copies for the tensor-core contractions, every one K-major
     // ([out][2 in]: hi | lo): W1, W2, Wr (forward), their transposes
     // (adjoint), Wqk.

@@ -1,71 +1,15 @@
-// Message-passing layer: edge embedding (Bessel x envelope, real SH),
+// Message-passing layers after the first (first.cu): edge embedding (Bessel x envelope, real SH),
 // segmented scatter-sum with one warp per receiver, and the adjoint (forces
 // and feature gradients): each pair's force once, from its lower atom, in
 // fixed point; each atom's sender-role gradient gathered over its row of the
 // symmetric neighbour list. Node-level MLP contractions: SIMT fp32 GEMM with
 // fused epilogues.
-#include <type_traits>
-
 #include "mp.cuh"
+#include "pack.cuh"
 
 namespace dmts {
 
 constexpr int MP_WARPS = 4;
-
-// ------------------------------------------------------------ channel packs
-// A lane owns CPW consecutive channels. With CPW even they are processed as
-// pairs in packed fp32 arithmetic (fma.rn.f32x2 / mul.rn.f32x2 of sm_100 and
-// later: one instruction issues two channels, each element rounded exactly as
-// fmaf / a plain product), with CPW = 1 as scalars. Quantities that multiply
-// every channel alike (radial basis, harmonics) are stored in shared memory
-// already duplicated into both halves of a pair.
-template <int CPW>
-struct Pack {
-    static constexpr int W = CPW % 2 == 0 ? 2 : 1;   // channels per pack
-    static constexpr int NP = CPW / W;               // packs per lane
-    using T = typename std::conditional<W == 2, float2, float>::type;
-};
-
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
-__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-__device__ __forceinline__ float vsub(float a, float b) { return a - b; }
-__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float vneg(float a) { return -a; }
-__device__ __forceinline__ float vsum(float2 v) { return v.x + v.y; }
-__device__ __forceinline__ float vsum(float v) { return v; }
-__device__ __forceinline__ float vget(float2 v, int h) { return h ? v.y : v.x; }
-__device__ __forceinline__ float vget(float v, int) { return v; }
-template <class T>
-__device__ __forceinline__ T vdup(float v) {
-    if constexpr (std::is_same<T, float2>::value) return make_float2(v, v);
-    else return v;
-}
-
-// CPW consecutive floats at p (aligned to 4 * CPW bytes) as packs, and back.
-template <int CPW, class T>
-__device__ __forceinline__ void ldp(const float *p, T *v) {
-    if constexpr (CPW == 4) {
-        const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = make_float2(t.x, t.y);
-        v[1] = make_float2(t.z, t.w);
-    } else if constexpr (CPW == 2) {
-        v[0] = __ldg(reinterpret_cast<const float2 *>(p));
-    } else {
-        v[0] = __ldg(p);
-    }
-}
-
-template <int CPW, class T>
-__device__ __forceinline__ void stp(float *p, const T *v) {
-    if constexpr (CPW == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
-    else if constexpr (CPW == 2) *reinterpret_cast<float2 *>(p) = v[0];
-    else *p = v[0];
-}
 
 // ------------------------------------------------------------------ forward
 // Warp per receiver i, lane owns CPW consecutive channels c = lane*CPW + u.
@@ -183,24 +127,6 @@ __global__ void __launch_bounds__(MP_WARPS * 32) k_mp_fwd(EdgeGeom g, LayerIO io
         }
         if (io.A) stp<CPW>(io.A + ((size_t)i * NLM + lm) * C + co + lane * CPW, a);
     }
-    if (LMAX >= 1 && io.V) {
-        // vector part of the tensor heads, V_h = sum_c U[h][c] A[l=1][c]
-        for (int h = 0; h < io.n_l; ++h) {
-            T u4[NP];
-            ldp<CPW>(io.U + (size_t)h * C + co + lane * CPW, u4);
-#pragma unroll
-            for (int cmp = 0; cmp < 3; ++cmp) {
-                float part = 0.f;
-#pragma unroll
-                for (int p = 0; p < NP; ++p)
-#pragma unroll
-                    for (int hh = 0; hh < PW; ++hh)
-                        part = fmaf(vget(u4[p], hh), io.nu * vget(acc[1 + cmp][p], hh), part);
-                part = warp_sum(part);
-                if (lane == 0) io.V[(size_t)i * nc_v_stride(io.n_l) + h * 3 + cmp] = part;
-            }
-        }
-    }
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
         stp<CPW>(io.q + (size_t)i * NL * C + l * C + co + lane * CPW, qv[l]);
@@ -229,7 +155,7 @@ __global__ void __launch_bounds__(MP_WARPS * 32) k_mp_fwd(EdgeGeom g, LayerIO io
 // with -, in 32.32 fixed point (exact, order-independent sums; every pair's
 // two terms cancel exactly), and so does its virial term. A lower
 // neighbour j < a contributes only its sender-role term to g_s_a (R, no R',
-// no force), and nothing in a layer without that gradient.
+// no force).
 //
 // Shared memory per block (one warp; 21.4 KB at C = 128, l_max = 2): 32 edge
 // records of packs (f_c B_k, its r-derivative, Y_lm) and of scalars
@@ -258,10 +184,7 @@ struct BwdSmem {
     static constexpr size_t bytes = r_bytes + ga_bytes + g_bytes + j_bytes + f_bytes;
 };
 
-// SG = false (io.gs_out == nullptr) skips the sender-role gradient: the
-// first layer's input features are the species embedding, constant in the
-// positions, so nothing consumes it there.
-template <int C, int LMAX, int K, bool VIR, bool SG>
+template <int C, int LMAX, int K, bool VIR>
 __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO io) {
     using S = BwdSmem<C, LMAX, K, VIR>;
     using T = typename S::T;
@@ -327,7 +250,7 @@ __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO i
         // warp owns): rows are ascending, so g_s_a takes its terms in row
         // order whatever the chunk boundaries (which move with the list's
         // skin entries)
-        const bool up = act && j > a, lo = SG && act && j < a;
+        const bool up = act && j > a, lo = act && j < a;
         const unsigned mu = __ballot_sync(DMTS_FULL, up), ml = __ballot_sync(DMTS_FULL, lo);
         const int n_up = __popc(mu), n_lo = __popc(ml);
         if (up || lo) {
@@ -361,32 +284,30 @@ __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO i
             sh_j[pos] = j;
         }
         __syncwarp();
-        if (SG) {
-            // lower neighbours: the sender-role gradient only
+        // lower neighbours: the sender-role gradient only
 #pragma unroll 2
-            for (int t = 0; t < n_lo; ++t) {
-                const int jt = sh_j[t];
-                const T *rec = sh_r[t];
-                T gj[NLM][NP];
+        for (int t = 0; t < n_lo; ++t) {
+            const int jt = sh_j[t];
+            const T *rec = sh_r[t];
+            T gj[NLM][NP];
 #pragma unroll
-                for (int lm = 0; lm < NLM; ++lm) ldp<CPW>(io.gA + ((size_t)jt * NLM + lm) * C + lane * CPW, gj[lm]);
+            for (int lm = 0; lm < NLM; ++lm) ldp<CPW>(io.gA + ((size_t)jt * NLM + lm) * C + lane * CPW, gj[lm]);
 #pragma unroll
-                for (int p = 0; p < NP; ++p) {
+            for (int p = 0; p < NP; ++p) {
 #pragma unroll
-                    for (int l = 0; l < NL; ++l) {
-                        T s0 = vdup<T>(0.f), s2 = vdup<T>(0.f);
+                for (int l = 0; l < NL; ++l) {
+                    T s0 = vdup<T>(0.f), s2 = vdup<T>(0.f);
 #pragma unroll
-                        for (int k = 0; k < K; k += 2) {
-                            s0 = vfma(W[l][k][p], rec[k], s0);
-                            s2 = vfma(W[l][k + 1][p], rec[k + 1], s2);
-                        }
-                        const T R = vadd(s0, s2);
-                        T wl = vdup<T>(0.f);
-#pragma unroll
-                        for (int lm = l * l; lm < (l + 1) * (l + 1); ++lm) wl = vfma(gj[lm][p], rec[2 * K + lm], wl);
-                        if (l & 1) gso[p] = vfma(R, wl, gso[p]);
-                        else gse[p] = vfma(R, wl, gse[p]);
+                    for (int k = 0; k < K; k += 2) {
+                        s0 = vfma(W[l][k][p], rec[k], s0);
+                        s2 = vfma(W[l][k + 1][p], rec[k + 1], s2);
                     }
+                    const T R = vadd(s0, s2);
+                    T wl = vdup<T>(0.f);
+#pragma unroll
+                    for (int lm = l * l; lm < (l + 1) * (l + 1); ++lm) wl = vfma(gj[lm][p], rec[2 * K + lm], wl);
+                    if (l & 1) gso[p] = vfma(R, wl, gso[p]);
+                    else gse[p] = vfma(R, wl, gse[p]);
                 }
             }
         }
@@ -433,13 +354,11 @@ __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO i
                             const T gam = vfma(sh_ga[lm][p * 32 + lane], sj[p], vmul(gj[lm][p], sas));
                             tl = vfma(gam, y[lm], tl);
                             beta[lm] = vfma(gam, R[l], beta[lm]);
-                            if (SG) wl = vfma(gj[lm][p], y[lm], wl);
+                            wl = vfma(gj[lm][p], y[lm], wl);
                         }
                         rho = vfma(Rp[l], tl, rho);
-                        if (SG) {
-                            if (l & 1) gso[p] = vfma(R[l], wl, gso[p]);
-                            else gse[p] = vfma(R[l], wl, gse[p]);
-                        }
+                        if (l & 1) gso[p] = vfma(R[l], wl, gso[p]);
+                        else gse[p] = vfma(R[l], wl, gse[p]);
                     }
                 }
                 // this lane's share (its channels) of the pair's force on a
@@ -524,7 +443,6 @@ __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO i
         fix_add(fa + 2, oa[2]);
         if (VIR) fix_add(io.Wfix + a, ow);
     }
-    if (!SG) return;
     T gin[NP], gout[NP];
     ldp<CPW>(io.gs_in + (size_t)a * C + lane * CPW, gin);
 #pragma unroll
@@ -567,51 +485,30 @@ void launch_fix_convert(int n, unsigned long long *Ffix, float *F, unsigned long
 
 // In the forward pass 128 channels are split over two blocks (64 per warp):
 // half the registers, twice the warps in flight to hide the neighbour loads.
-// The tensor-head vectors V sum over all channels, so a launch that writes V
-// keeps the channels in one warp.
 template <int C, int LMAX>
 static void fwd_c(const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
     constexpr int SP = C >= 128 ? 2 : 1;
     const int blocks = (g.n_atoms + MP_WARPS - 1) / MP_WARPS;
-    if (SP > 1 && !io.V)
-        k_mp_fwd<C, LMAX, 8, SP><<<dim3(blocks, SP), MP_WARPS * 32, 0, st>>>(g, io);
-    else
-        k_mp_fwd<C, LMAX, 8, 1><<<blocks, MP_WARPS * 32, 0, st>>>(g, io);
+    k_mp_fwd<C, LMAX, 8, SP><<<dim3(blocks, SP), MP_WARPS * 32, 0, st>>>(g, io);
     count_launch();
 }
 
-template <int C, int LMAX, bool VIR, bool SG>
+template <int C, int LMAX, bool VIR>
 static void bwd_launch(const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
     constexpr size_t smem = BwdSmem<C, LMAX, 8, VIR>::bytes;
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_mp_bwd<C, LMAX, 8, VIR, SG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_mp_bwd<C, LMAX, 8, VIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int blocks = (g.n_atoms + BWD_WARPS - 1) / BWD_WARPS;
-    k_mp_bwd<C, LMAX, 8, VIR, SG><<<blocks, BWD_WARPS * 32, smem, st>>>(g, io);
+    k_mp_bwd<C, LMAX, 8, VIR><<<blocks, BWD_WARPS * 32, smem, st>>>(g, io);
     count_launch();
 }
 
-// The virial variant (io.Wfix set) and the variant without the sender-role
-// gradient (io.gs_out null) are separate instantiations, so that each
-// carries no register or instruction it does not use.
+// The virial variant (io.Wfix set) is a separate instantiation, so that the
+// other carries no register or instruction it does not use.
 template <int C, int LMAX>
 static void bwd_c(const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
-    const bool gs = io.gs_out != nullptr;
-    if (io.Wfix) gs ? bwd_launch<C, LMAX, true, true>(g, io, st) : bwd_launch<C, LMAX, true, false>(g, io, st);
-    else gs ? bwd_launch<C, LMAX, false, true>(g, io, st) : bwd_launch<C, LMAX, false, false>(g, io, st);
+    io.Wfix ? bwd_launch<C, LMAX, true>(g, io, st) : bwd_launch<C, LMAX, false>(g, io, st);
 }
-
-#define DMTS_DISPATCH(FN, C, LMAX, ...)                          \
-    do {                                                         \
-        if ((C) == 32 && (LMAX) == 0) FN<32, 0>(__VA_ARGS__);    \
-        else if ((C) == 32 && (LMAX) == 1) FN<32, 1>(__VA_ARGS__); \
-        else if ((C) == 32 && (LMAX) == 2) FN<32, 2>(__VA_ARGS__); \
-        else if ((C) == 64 && (LMAX) == 0) FN<64, 0>(__VA_ARGS__); \
-        else if ((C) == 64 && (LMAX) == 1) FN<64, 1>(__VA_ARGS__); \
-        else if ((C) == 64 && (LMAX) == 2) FN<64, 2>(__VA_ARGS__); \
-        else if ((C) == 128 && (LMAX) == 0) FN<128, 0>(__VA_ARGS__); \
-        else if ((C) == 128 && (LMAX) == 1) FN<128, 1>(__VA_ARGS__); \
-        else if ((C) == 128 && (LMAX) == 2) FN<128, 2>(__VA_ARGS__); \
-    } while (0)
 
 void launch_mp_fwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
     (void)K;

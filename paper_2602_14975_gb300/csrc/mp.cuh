@@ -26,12 +26,9 @@ struct LayerIO {
     float *A;                // [N][NLM][C]  (forward out; nullable: not stored)
     float *q;                // [N][(LMAX+1)C] (forward out, fp32)
     __nv_bfloat16 *q_bf16;   // optional split-bf16 copy of q, [N][2(LMAX+1)C] (forward out)
-    const float *U;          // optional: tensor-head mix U[n_l][C] (NC embedding)
-    float *V;                // optional: V[N][nc_v_stride(n_l)], V[i][3h + a] = sum_c U[h][c] A[1+a][c]
-    int n_l;
     const float *gA;         // [N][NLM][C]  (backward in)
     const float *gs_in;      // [N][C]       (backward in)
-    float *gs_out;           // [N][C]       (backward out; nullable: not computed)
+    float *gs_out;           // [N][C]       (backward out)
     __nv_bfloat16 *gs_out_bf16;  // optional split-bf16 copy of gs_out, [N][2C]
     unsigned long long *Ffix;  // [N][3] (backward): forces added in 32.32 fixed point
     unsigned long long *Wfix;  // [N] (backward, nullable): per-atom virial proxy, pair form, fixed point
@@ -68,12 +65,48 @@ __device__ __forceinline__ void stv(float *p, const float *v) {
     }
 }
 
+// First layer (input features = the species embedding), first.cu.
+struct FirstIO {
+    const uint8_t *species;  // [N] codes 0..n_species-1
+    const float *emb;        // [n_species][C]
+    const float *wrad;       // [L+1][K][C]
+    int n_species;           // <= DMTS_MAX_SPECIES
+    float nu;
+    float *A;                // [N][NLM][C] (forward out, nullable: not stored; backward in)
+    float *q;                // [N][(LMAX+1)C] (forward out, nullable)
+    __nv_bfloat16 *q_bf16;   // optional split-bf16 copy of q (forward out)
+    const float *UW;         // tensor-head weights [n_l][n_species][K] (with V)
+    float *V;                // optional: tensor-head vectors [N][nc_v_stride(n_l)]
+    int n_l;
+    const float *gq;         // [N][(LMAX+1)C] dU/dq (backward in)
+    unsigned long long *Ffix, *Wfix;   // as LayerIO
+    int *err;
+};
+
+#define DMTS_DISPATCH(FN, C, LMAX, ...)                          \
+    do {                                                         \
+        if ((C) == 32 && (LMAX) == 0) FN<32, 0>(__VA_ARGS__);    \
+        else if ((C) == 32 && (LMAX) == 1) FN<32, 1>(__VA_ARGS__); \
+        else if ((C) == 32 && (LMAX) == 2) FN<32, 2>(__VA_ARGS__); \
+        else if ((C) == 64 && (LMAX) == 0) FN<64, 0>(__VA_ARGS__); \
+        else if ((C) == 64 && (LMAX) == 1) FN<64, 1>(__VA_ARGS__); \
+        else if ((C) == 64 && (LMAX) == 2) FN<64, 2>(__VA_ARGS__); \
+        else if ((C) == 128 && (LMAX) == 0) FN<128, 0>(__VA_ARGS__); \
+        else if ((C) == 128 && (LMAX) == 1) FN<128, 1>(__VA_ARGS__); \
+        else if ((C) == 128 && (LMAX) == 2) FN<128, 2>(__VA_ARGS__); \
+    } while (0)
+
+// UW[h][z][k] = sum_c U[h][c] emb[z][c] wrad[1][k][c], of the model alone.
+void launch_tensor_head_weights(int C, int S, int n_l, const float *emb, const float *wrad, const float *U, float *UW,
+                                cudaStream_t st);
+void launch_first_fwd(int C, int lmax, const EdgeGeom &g, const FirstIO &io, cudaStream_t st);
+void launch_first_bwd(int C, int lmax, const EdgeGeom &g, const FirstIO &io, cudaStream_t st);
+
 void launch_mp_fwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io, cudaStream_t st);
 // The forward layer with the radial contraction R = W B on the tensor cores
-// (split-bf16 operands, nseg as for launch_gemm_tc): C = 128, K = 8 and no
-// tensor-head output (io.V null) only; err receives DMTS_E_TIMEOUT if a
+// (split-bf16 operands, nseg as for launch_gemm_tc): C = 128 and K = 8 only; err receives DMTS_E_TIMEOUT if a
 // bounded wait on the tensor cores runs out.
-bool mp_fwd_tc_supported(int C, int K, const LayerIO &io);
+bool mp_fwd_tc_supported(int C, int K);
 void launch_mp_fwd_tc(int lmax, const EdgeGeom &g, const LayerIO &io, int nseg, int *err, cudaStream_t st);
 void launch_mp_bwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io, cudaStream_t st);
 // The adjoint's fixed-point forces (and virial, Wfix nullable) -> fp32 F and

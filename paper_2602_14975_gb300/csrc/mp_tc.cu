@@ -332,7 +332,7 @@ int resident_ctas(const void *fn, int threads, size_t dyn_smem, int dev) {
     return std::max(n, 1);
 }
 
-bool mp_fwd_tc_supported(int C, int K, const LayerIO &io) { return C == TF_C && K == TF_K && !io.V; }
+bool mp_fwd_tc_supported(int C, int K) { return C == TF_C && K == TF_K; }
 
 void launch_mp_fwd_tc(int lmax, const EdgeGeom &g, const LayerIO &io, int nseg, int *err, cudaStream_t st) {
     if (g.n_atoms == 0) return;
