@@ -42,12 +42,10 @@ KCAL_A3_PER_ATM = 101325.0 * 6.02214076e23 * 1e-30 / 4184.0   # 1 atm in kcal/mo
 
 NCU_TRAFFIC = {
     "mp_bwd": {"bytes_per_launch": (154229760 + 19248896 + 154260992 + 16390400 + 139650304 + 268544) / 3,
-               # the adjoint's code: channel-pack helpers, kernel and launch, the
-               # argument structs, the device helpers
-               "sources": [("paper_2602_14975_gb300/csrc/mp.cu", ("// ---- channel packs", "// ---- forward")),
+               # the adjoint's code: channel-pack helpers, kernel, the argument
+               # structs, the device helpers
+               "sources": [("paper_2602_14975_gb300/csrc/pack.cuh", None),
                            ("paper_2602_14975_gb300/csrc/mp.cu", ("// ---- adjoint", "// In the forward pass")),
-                           ("paper_2602_14975_gb300/csrc/mp.cu", ("template <int C, int LMAX, bool VIR, bool SG>",
-                                                                  "#define DMTS_DISPATCH")),
                            ("paper_2602_14975_gb300/csrc/mp.cuh", ("struct EdgeGeom {", "template <int CPW>")),
                            ("paper_2602_14975_gb300/csrc/common.cuh", None)],
                "sha256": "8c1a3a7c5d60e748369169f7e9198032650ff7e2427e60f09026a2b70bc7c32c"},
