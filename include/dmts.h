@@ -56,10 +56,8 @@ typedef enum {
 } dmts_status;
 
 /*
- * Arithmetic of the MLP contractions, and of the per-edge radial
- * contraction R_lc = sum_k W_lkc f_c B_k of a conservative model with
- * C = 128 (the paper states none; the stand-in models run them as
- * follows). DMTS_FP32: fp32 SIMT products. DMTS_BF16:
+ * Arithmetic of the MLP contractions (the paper states none; the stand-in
+ * models run them as follows). DMTS_FP32: fp32 SIMT products. DMTS_BF16:
  * tensor cores, bf16 x bf16 products accumulated in fp32, each operand held
  * as a split pair hi = rn_bf16(v), lo = rn_bf16(v - hi) and the products
  * hi*hi + lo*hi + hi*lo accumulated (about 16 significant bits per operand;
@@ -67,6 +65,10 @@ typedef enum {
  * kernels with the hi*hi products only (one bf16 rounding per operand,
  * a third of the tensor-core work; forces off by a few per cent of the
  * message-passing force's RMS).
+ * With DMTS_BF16 and DMTS_BF16_PLAIN the neighbour sums of a conservative
+ * model's layers after the first run on the tensor cores too where C = 128,
+ * with operands split into fp16 pairs of 22 significant bits; all other
+ * neighbour sums are packed fp32.
  */
 typedef enum { DMTS_FP32 = 0, DMTS_BF16 = 1, DMTS_BF16_PLAIN = 2 } dmts_precision;
 

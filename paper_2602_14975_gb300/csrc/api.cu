@@ -294,10 +294,19 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
         !w.q.ensure(sizeof(float) * nc_ * NL) || !w.h.ensure(sizeof(float) * nc_ * L) ||
         !w.act.ensure(sizeof(float) * nc_) || !w.u.ensure(sizeof(float) * nc_) || !w.gz.ensure(sizeof(float) * nc_) ||
         !w.gs0.ensure(sizeof(float) * nc_) || !w.gs1.ensure(sizeof(float) * nc_) ||
-        !w.gA.ensure(sizeof(float) * nc_ * NLM) || !w.e_atom.ensure(sizeof(float) * (N + 1)) ||
+        !w.e_atom.ensure(sizeof(float) * (N + 1)) ||
         !w.ftmp.ensure(sizeof(float) * 3 * (N + 1)) || (virial && !w.cons_w.ensure(sizeof(float) * (N + 1))) ||
         (forces && !ensure_zeroed(ctx, w.cons_ffix, sizeof(unsigned long long) * 3 * (N + 1), st)) ||
         (forces && virial && !ensure_zeroed(ctx, w.cons_wfix, sizeof(unsigned long long) * (N + 1), st)))
+        return fail(ctx, DMTS_E_OOM, "workspace allocation failed");
+    // layers after the first on the tensor cores, for models that run their
+    // contractions there (against 64 bits the message-passing force's error is
+    // 1.6e-5 of its norm then, 1.8e-5 with the radial products split in bf16;
+    // an fp32 model's would grow from 1.6e-6 to 2.1e-6)
+    const bool tc = bf && mp_tc_supported(C, m.K);
+    if (tc && L > 1 && (!w.s16.ensure(4 * nc_) || !w.s_exp.ensure(sizeof(int) * (size_t)N)))
+        return fail(ctx, DMTS_E_OOM, "workspace allocation failed");
+    if (L > 1 && forces && !w.gA.ensure(sizeof(float) * nc_ * NLM))
         return fail(ctx, DMTS_E_OOM, "workspace allocation failed");
     // split-bf16 copies: 4 bytes per logical element (hi and lo)
     if (bf && (!w.q_bf.ensure(4 * nc_ * NL + 16) || !w.act_bf.ensure(4 * nc_ + 16) || !w.s_bf.ensure(4 * nc_ + 16) ||
@@ -331,8 +340,15 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
             launch_first_fwd(C, m.lmax, g, f, st);
         } else {
             ProfScope ps(ctx, "mp_fwd", st);
-            if (bf && mp_fwd_tc_supported(C, m.K)) launch_mp_fwd_tc(m.lmax, g, io, m.nseg, ctx->d_err, st);
-            else launch_mp_fwd(C, m.lmax, m.K, g, io, st);
+            if (tc) {
+                io.s16 = (const __half *)w.s16.p;
+                io.s_exp = (const int *)w.s_exp.p;
+                io.q = nullptr;                 // the tensor-core contraction reads only the split-bf16 copy
+                launch_feature_split(N, io.s, (void *)io.s16, (int *)io.s_exp, st);
+                launch_mp_fwd_tc(m.lmax, g, io, ctx->d_err, st);
+            } else {
+                launch_mp_fwd(C, m.lmax, m.K, g, io, st);
+            }
         }
         Epi e1 = epi(EPI_BIAS_SILU);
         e1.bias = m.b1[t];

@@ -72,6 +72,14 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
+// Sum of a 64-bit integer over the warp (modulo 2^64), in every lane: three
+// 32-bit reductions, of its upper half and the two quarters of its lower half.
+__device__ __forceinline__ long long warp_sum_fix(long long v) {
+    const int hi = __reduce_add_sync(DMTS_FULL, (int)(v >> 32));
+    const unsigned m = __reduce_add_sync(DMTS_FULL, (unsigned)v >> 16), lo = __reduce_add_sync(DMTS_FULL, (unsigned)v & 0xffffu);
+    return ((long long)hi << 32) + ((long long)m << 16) + (long long)lo;
+}
+
 // Replica of an atom from the replica offsets (binary search, R small).
 __device__ __forceinline__ int replica_of(const int *rep_off, int n_rep, int atom) {
     int lo = 0, hi = n_rep - 1;

@@ -23,6 +23,7 @@
 // the general layers (mp.cu, mp_tc.cu) after it.
 #include <algorithm>
 
+#include "edge.cuh"
 #include "mp.cuh"
 #include "pack.cuh"
 
@@ -37,37 +38,6 @@ constexpr int FL_K = 8;      // radial functions: lane = (k, g), k = lane % 8
 // that no sum depends on the skin entries a list happens to hold.
 constexpr int FL_UNIT = 3;      // candidates per lane and sweep step, loaded together
 constexpr int FL_QUEUE = 128;   // at most 31 + 96 wait
-
-struct AtomGeom {
-    float x, y, z, bx, by, bz, ibx, iby, ibz;
-};
-
-// The wi-th atom in processing order: index, row bounds, position and box.
-struct Row {
-    int i, beg, end;
-    AtomGeom a;
-};
-
-__device__ __forceinline__ Row load_row(const EdgeGeom &g, int wi) {
-    Row r;
-    r.i = r.beg = r.end = 0;
-    if (wi >= g.n_atoms) return r;
-    const int i = g.order ? __ldg(g.order + wi) : wi;
-    const int rep = g.atom_rep[i];
-    r.i = i;
-    r.beg = g.row_ptr[i];
-    r.end = g.row_ptr[i + 1];
-    r.a.x = g.x[3 * i]; r.a.y = g.x[3 * i + 1]; r.a.z = g.x[3 * i + 2];
-    r.a.bx = g.box[3 * rep]; r.a.by = g.box[3 * rep + 1]; r.a.bz = g.box[3 * rep + 2];
-    return r;
-}
-
-__device__ __forceinline__ AtomGeom wrap_inverse(AtomGeom a) {
-    a.ibx = a.bx > 0.f ? 1.f / a.bx : 0.f;
-    a.iby = a.by > 0.f ? 1.f / a.by : 0.f;
-    a.ibz = a.bz > 0.f ? 1.f / a.bz : 0.f;
-    return a;
-}
 
 // Sweeps the row [beg, end): batch(n) is called with n <= 32 queued edges,
 // the e-th at queue[(taken + e) % 64] (displacement; w: 8 j + species).
@@ -460,13 +430,10 @@ __global__ void __launch_bounds__(256, 2) k_first_bwd(EdgeGeom g, FirstIO io) {
             }
             __syncwarp();   // Q and queue slots read before they are overwritten
         });
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ox += __shfl_xor_sync(DMTS_FULL, ox, o);
-            oy += __shfl_xor_sync(DMTS_FULL, oy, o);
-            oz += __shfl_xor_sync(DMTS_FULL, oz, o);
-            if (VIR) ow += __shfl_xor_sync(DMTS_FULL, ow, o);
-        }
+        ox = warp_sum_fix(ox);
+        oy = warp_sum_fix(oy);
+        oz = warp_sum_fix(oz);
+        if (VIR) ow = warp_sum_fix(ow);
         if (lane == 0) {
             unsigned long long *fa = io.Ffix + 3 * (size_t)i;
             fix_add(fa, ox);

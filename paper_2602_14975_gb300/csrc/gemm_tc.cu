@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256) k_gemm_tc(const __grid_constant__ CUtenso
             const uint32_t sa = base + s * stage_bytes, sb = sa + a_bytes;
 #pragma unroll
             for (int kk = 0; kk < TC_K / 16; ++kk)
-                mma_bf16(tmem, smem_desc(sa + kk * 32), smem_desc(sb + kk * 32), idesc, (k > 0 || kk > 0) ? 1u : 0u);
+                mma_f16kind(tmem, smem_desc(sa + kk * 32), smem_desc(sb + kk * 32), idesc, (k > 0 || kk > 0) ? 1u : 0u);
             mma_commit(smem_u32(&bar_empty[s]));
         }
         consumed_sh = k;   // stages whose loads landed

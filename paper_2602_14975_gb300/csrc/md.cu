@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(NCH_WARPS * 32) k_nc_head(NCHeadArgs g) {
             if (lane == 0) set_error(g.err, DMTS_E_NONFINITE);
             return;
         }
-        ox = seg_sum_ll(ox, 0); oy = seg_sum_ll(oy, 0); oz = seg_sum_ll(oz, 0);
+        ox = warp_sum_fix(ox); oy = warp_sum_fix(oy); oz = warp_sum_fix(oz);
         if (g.W) w = warp_sum(w);
         if (lane == 0) {
             unsigned long long *fa = g.Ffix + 3 * (size_t)a;

@@ -9,6 +9,7 @@
 #include "epilogue.cuh"
 #include "mp.cuh"
 #include "pack.cuh"
+#include "ptx.cuh"
 
 namespace dmts {
 
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(MP_WARPS * 32) k_mp_fwd(EdgeGeom g, LayerIO io
             a[p] = vmul(nu, acc[lm][p]);
             qv[l][p] = vfma(a[p], a[p], qv[l][p]);
         }
-        if (io.A) stp<CPW>(io.A + ((size_t)i * NLM + lm) * C + co + lane * CPW, a);
+        stp<CPW>(io.A + ((size_t)i * NLM + lm) * C + co + lane * CPW, a);
     }
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
@@ -431,13 +432,10 @@ __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO i
         __syncwarp();
     }
     // a's side: the integer sums of the lanes that added up its pairs
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        oa[0] += __shfl_xor_sync(DMTS_FULL, oa[0], o);
-        oa[1] += __shfl_xor_sync(DMTS_FULL, oa[1], o);
-        oa[2] += __shfl_xor_sync(DMTS_FULL, oa[2], o);
-        if (VIR) ow += __shfl_xor_sync(DMTS_FULL, ow, o);
-    }
+    oa[0] = warp_sum_fix(oa[0]);
+    oa[1] = warp_sum_fix(oa[1]);
+    oa[2] = warp_sum_fix(oa[2]);
+    if (VIR) ow = warp_sum_fix(ow);
     if (__any_sync(DMTS_FULL, bad) && lane == 0) set_error(io.err, (int)DMTS_E_NONFINITE);
     if (lane == 0) {
         unsigned long long *fa = io.Ffix + 3 * (size_t)a;
@@ -540,11 +538,6 @@ void launch_mp_bwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io,
 // accesses. At 192 rows it is bound by latency: 17 -> 7.5 us per call.
 constexpr int GEMM_KC = 32, GEMM_LD = GEMM_KC + 4, GEMM_STAGES = 3;
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok) {
-    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
-
 template <int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_f32(int M, int N, int K, const float *__restrict__ Act,
                                                                    const float *__restrict__ W, int trans, int vec, Epi e) {
@@ -561,13 +554,13 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_f32(int M, int N
         for (int q = tid; q < BM * CH; q += THREADS) {
             const int r = q / CH, k = k0 + 4 * (q % CH);
             const bool ok = m0 + r < M && k < K;
-            cp_async16(a + r * GEMM_LD + 4 * (q % CH), ok ? Act + (size_t)(m0 + r) * K + k : Act, ok);
+            cp_async16(smem_u32(a + r * GEMM_LD + 4 * (q % CH)), ok ? Act + (size_t)(m0 + r) * K + k : Act, ok);
         }
         if (trans) {
             for (int q = tid; q < BN * CH; q += THREADS) {
                 const int r = q / CH, k = k0 + 4 * (q % CH);
                 const bool ok = n0 + r < N && k < K;
-                cp_async16(b + r * GEMM_LD + 4 * (q % CH), ok ? W + (size_t)(n0 + r) * K + k : W, ok);
+                cp_async16(smem_u32(b + r * GEMM_LD + 4 * (q % CH)), ok ? W + (size_t)(n0 + r) * K + k : W, ok);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -637,7 +630,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_f32(int M, int N
     }
     // the tile through shared memory, so that the epilogue's accesses are
     // whole rows whatever its mode
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    cp_async_wait_all();
     __syncthreads();
     constexpr int LD = BN + 1;
     static_assert(BM * LD <= GEMM_STAGES * (BM + BN) * GEMM_LD, "the staged tile reuses the pipeline buffers");

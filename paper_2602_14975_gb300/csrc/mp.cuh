@@ -1,6 +1,8 @@
 // Kernels of the message-passing layer (edge embedding + segmented
 // scatter-sum) and of its adjoint, plus the node-level GEMMs of the MLPs.
 #pragma once
+#include <cuda_fp16.h>
+
 #include "common.cuh"
 
 namespace dmts {
@@ -21,10 +23,12 @@ struct EdgeGeom {
 // Node-level arrays for one layer.
 struct LayerIO {
     const float *s;          // [N][C] input features s^t
+    const __half *s16;       // split-fp16 copy of s and its row exponents (tensor-core layers)
+    const int *s_exp;
     const float *wrad;       // [L+1][K][C]
     float nu;
-    float *A;                // [N][NLM][C]  (forward out; nullable: not stored)
-    float *q;                // [N][(LMAX+1)C] (forward out, fp32)
+    float *A;                // [N][NLM][C]  (forward out)
+    float *q;                // [N][(LMAX+1)C] (forward out, fp32; nullable in the tensor-core layers)
     __nv_bfloat16 *q_bf16;   // optional split-bf16 copy of q, [N][2(LMAX+1)C] (forward out)
     const float *gA;         // [N][NLM][C]  (backward in)
     const float *gs_in;      // [N][C]       (backward in)
@@ -103,11 +107,14 @@ void launch_first_fwd(int C, int lmax, const EdgeGeom &g, const FirstIO &io, cud
 void launch_first_bwd(int C, int lmax, const EdgeGeom &g, const FirstIO &io, cudaStream_t st);
 
 void launch_mp_fwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io, cudaStream_t st);
-// The forward layer with the radial contraction R = W B on the tensor cores
-// (split-bf16 operands, nseg as for launch_gemm_tc): C = 128 and K = 8 only; err receives DMTS_E_TIMEOUT if a
-// bounded wait on the tensor cores runs out.
-bool mp_fwd_tc_supported(int C, int K);
-void launch_mp_fwd_tc(int lmax, const EdgeGeom &g, const LayerIO &io, int nseg, int *err, cudaStream_t st);
+// The layers after the first on the tensor cores (mp_tc.cu; C = 128 and K = 8
+// only): the neighbour sums as products with split-fp16 operands. s16 and
+// s_exp hold the features' split copy ([N][2C] fp16 and one exponent per
+// row, launch_feature_split). err receives DMTS_E_TIMEOUT if a bounded wait
+// on the tensor cores runs out.
+bool mp_tc_supported(int C, int K);
+void launch_feature_split(int n, const float *s, void *s16, int *s_exp, cudaStream_t st);
+void launch_mp_fwd_tc(int lmax, const EdgeGeom &g, const LayerIO &io, int *err, cudaStream_t st);
 void launch_mp_bwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io, cudaStream_t st);
 // The adjoint's fixed-point forces (and virial, Wfix nullable) -> fp32 F and
 // W, the fixed-point words cleared for the next evaluation.

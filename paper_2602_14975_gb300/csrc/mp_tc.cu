@@ -1,33 +1,23 @@
-// Forward message-passing layer with the radial contraction on the tensor
-// cores (models with split-bf16 contractions, C = 128 channels, K = 8).
+// Message-passing layers after the first on the tensor cores (models that run
+// their contractions there, C = 128 channels).
 //
-// For receiver i and each active edge e = (i, j) the layer needs
-//   R_lc(e) = sum_k W_lkc f_c(r) B_k(r)                       (radial)
-//   A_i[lm][c] = nu sum_e R_lc(e) s_j[c] Y_lm(e)              (messages)
-// The radial contraction is a product of the layer's [C x K] weights with
-// the edges' [K] basis vectors: one tcgen05.mma per l with the C = 128
-// channels as the M = 128 rows (TMEM lanes) and 32 edges as N columns. The
-// rest runs on the CUDA cores with one thread per channel (thread t reads
-// TMEM lane t), two edges at a time in packed fp32.
+// With E_ij[lm,k] = f_c(r) B_k(r) Y_lm(n) of an edge (receiver i, neighbour j)
+// the layer is, per receiver,
+//   T_i[lm,k][c] = sum_j E_ij[lm,k] s_j[c],   A_i[lm][c] = nu sum_k W_lkc T_i[lm,k][c]:
+// the neighbour sum is a dense product [C x neighbours] x [neighbours x (lm,k)]
+// for tcgen05, and the radial weights are applied once per atom instead of
+// once per edge.
 //
-// Operands are split-bf16 (common.cuh) and concatenated along K, so one
-// K = 32 product holds hi*hi + lo*hi + hi*lo:
-//   A row c (weights): W_hi[0..7] | W_lo[0..7] | W_hi[0..7] | 0
-//   B row e (edge):    b_hi[0..7] | b_hi[0..7] | b_lo[0..7] | 0
-// (nseg = 1 keeps W_hi alone: hi*hi only). Rows are 128-byte-swizzled
-// K-major tiles: l = 0 and 1 share a weight tile (bytes 0-63 and 64-127 of
-// each row, two K = 16 steps each), and every basis row holds the edge's
-// 64 bytes twice, so that each l's MMA starts at its own half.
-//
-// One CTA of 128 threads (four per SM) owns a TMEM accumulator of 128
-// columns and processes receivers in cell order (grid-stride). Per
-// receiver, 96 candidates of its row at a time are tested; the active ones
-// are compacted into shared memory (basis row for the MMA, Y_lm, neighbour
-// index), then each chunk of 32 is contracted and consumed. Every mbarrier wait is
-// bounded: on timeout the CTA records DMTS_E_TIMEOUT, waits (bounded) for
-// the MMAs it issued, frees its tensor memory and returns.
+// Operands are split-fp16: v 2^n = hi + lo with hi = rn_fp16, lo = rn_fp16(v 2^n - hi)
+// (22 significant bits), and hi*hi + lo*hi + hi*lo is accumulated in fp32. The
+// power of two n puts a row's largest element just below 2^14, so that any
+// feature range fits; scaling is exact and undone on the results.
 #include <algorithm>
+#include <climits>
+#include <cmath>
+#include <cuda_fp16.h>
 
+#include "edge.cuh"
 #include "mp.cuh"
 #include "ptx.cuh"
 #include "tc.cuh"
@@ -36,279 +26,535 @@ namespace dmts {
 
 namespace {
 
-constexpr int TF_C = 128;        // channels = TMEM lanes = threads per CTA
-constexpr int TF_K = 8;          // radial basis functions
-constexpr int TF_PASS = 96;      // candidates tested per pass (one per thread of the first three warps)
-constexpr int TF_CHUNK = 32;     // edges per MMA (N)
-constexpr int TF_TMEM = 128;     // TMEM columns: (l_max + 1) x 32 <= 96
+constexpr int TC_C = 128;        // channels = TMEM lanes
+constexpr int TC_KR = 8;         // radial functions
+constexpr int TC_E = 64;         // edges per chunk
+
+// Exponent n of a row scale: 2^n maps values below 2 * 2^e into fp16's upper
+// range; e is kept where 2^n and its inverse are normal floats.
+__device__ __forceinline__ int row_exponent(unsigned max_bits) {
+    return min(max((int)(max_bits >> 23) - 127, -100), 100);
+}
+__device__ __forceinline__ float pow2f(int n) { return __int_as_float((127 + n) << 23); }
+constexpr int TC_TOP = 13;       // scaled rows lie below 2^(TC_TOP + 1)
+
+__device__ __forceinline__ uint32_t h2u(__half2 v) { return *reinterpret_cast<uint32_t *>(&v); }
+
+// Split pair of two values.
+__device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &lo) {
+    const __half2 h = __floats2half2_rn(a, b);
+    const float2 f = __half22float2(h);
+    hi = h2u(h);
+    lo = h2u(__floats2half2_rn(a - f.x, b - f.y));
+}
+// Split pair of the products a y (lo: of the unrounded product).
+__device__ __forceinline__ void split2_prod(float2 a, float2 y, uint32_t &hi, uint32_t &lo) {
+    const float2 v = __fmul2_rn(a, y);
+    const __half2 h = __floats2half2_rn(v.x, v.y);
+    const float2 f = __half22float2(h);
+    const float2 r = __ffma2_rn(a, y, make_float2(-f.x, -f.y));
+    hi = h2u(h);
+    lo = h2u(__floats2half2_rn(r.x, r.y));
+}
+
+// Shared-memory tiles of a chunk:
+//  S (neighbour features): [hi | lo][2 channel blocks][64 edges][128 bytes], 128-byte swizzle;
+//  E (basis): [hi | lo][NB blocks of 16 (lm,k)][64 edges][32 bytes], 32-byte swizzle.
+constexpr uint32_t S_BLK = TC_E * 128, S_PART = 2 * S_BLK, S_BYTES = 2 * S_PART;
+constexpr uint32_t E_BLK = TC_E * 32;
 
 template <int LMAX>
-struct FwdTcSmem {
-    static constexpr int NL = LMAX + 1;
-    // weights: l = 2j and 2j + 1 share tile j (K-chunks 0-3 and 4-7 of its 128-byte rows)
-    static constexpr uint32_t a_bytes = ((NL + 1) / 2) * TF_C * 128;
-    static constexpr uint32_t b_bytes = TF_PASS * 128;        // basis rows of one pass
-    static constexpr size_t bytes = a_bytes + b_bytes + 1024;  // + alignment slack
+struct TcDims {
+    static constexpr int NL = LMAX + 1, NLM = NL * NL;
+    static constexpr int NK = NLM * TC_KR;                 // (lm, k) columns used
+    static constexpr int NB = (NK + 15) / 16, NN = NB * 16;   // blocks of 16, padded columns
+    static constexpr uint32_t e_part = NB * E_BLK, e_bytes = 2 * e_part;
 };
 
-__device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 a, __nv_bfloat16 b) {
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+// A bounded wait with one answer for the warp.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
+    return __all_sync(DMTS_FULL, mbar_wait(bar, parity)) != 0;
 }
 
-// Writes the 16-byte chunk j of row r of a swizzled tile.
-__device__ __forceinline__ void st_chunk(uint8_t *tile, int r, int j, uint4 v) {
-    *reinterpret_cast<uint4 *>(tile + swz128(r, j)) = v;
+// ---------------------------------------------------------------- front end
+// A CTA's work comes in chunks of up to 64 active edges of one receiver (the
+// g-th active edge of a row is slot g % 64 of chunk g / 64, whatever skin
+// entries the list holds); a row without active edges is one empty chunk. One
+// warp prepares them a chunk ahead of the others: it walks the rows, tests the
+// candidates (96 in flight), compacts the active ones and announces the chunk.
+constexpr int TC_COMPUTE = 256, TC_THREADS = TC_COMPUTE + 32;   // eight working warps and the front end
+constexpr int TC_PROD = 192;                                    // threads that form products (warps 0, 1, 4-7)
+
+struct Chunk {
+    int i, n, first, last;   // receiver (-1: no more chunks), edges, first / last chunk of its row
+    int e_ref;               // largest row exponent of the row's neighbours
+};
+
+struct FrontSmem {
+    uint64_t full[2];              // chunk announced
+    Chunk chunk[2];
+    alignas(16) float4 qd[2][TC_E];   // displacement, neighbour index
+    int qe[2][TC_E];                  // neighbour's row exponent
+};
+
+__device__ __forceinline__ void front_init(FrontSmem &f) {
+    mbar_init(smem_u32(&f.full[0]), 1);
+    mbar_init(smem_u32(&f.full[1]), 1);
 }
 
-__device__ __forceinline__ uint4 pack8(const __nv_bfloat16 *v) {
-    return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
-                      pack_bf16x2(v[6], v[7]));
-}
-
-template <int LMAX>
-__global__ void __launch_bounds__(TF_C, 4) k_mp_fwd_tc(EdgeGeom g, LayerIO io, int nseg, int *err) {
-    using SM = FwdTcSmem<LMAX>;
-    constexpr int NL = LMAX + 1, NLM = NL * NL, C = TF_C, K = TF_K;
-    extern __shared__ uint8_t tf_smem[];
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ uint32_t tmem_sh;
-    __shared__ int wcnt[TF_C / 32];
-    __shared__ __align__(16) int sJ[TF_PASS];
-    __shared__ __align__(16) float4 cd[TF_PASS];   // candidate displacement and r^2
-    __shared__ int cj[TF_PASS], perm[TF_PASS];
-    __shared__ __align__(16) float sY[NLM][TF_PASS];
-    __shared__ int err0;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t raw = smem_u32(tf_smem);
-    const uint32_t base = (raw + 1023u) & ~1023u;
-    uint8_t *pA = tf_smem + (base - raw), *pB = pA + SM::a_bytes;
-    const uint32_t sA = base, sB = base + SM::a_bytes;
-
-    if (tid == 0) {
-        mbar_init(smem_u32(&bar), 1);
-        mbar_init_fence();
-        err0 = *io.err;
+// bar_free completes once per chunk, when nothing reads its queue any more.
+// Returns false on a timeout.
+__device__ __forceinline__ bool front_end(const EdgeGeom &g, const LayerIO &io, FrontSmem &f, uint32_t bar_free,
+                                          int lane) {
+    constexpr int U = 3;
+    const int stride = gridDim.x;
+    const float rc2 = g.rc * g.rc;
+    auto index = [&](int wi) { return wi < g.n_atoms ? (g.order ? __ldg(g.order + wi) : wi) : -1; };
+    // staged so that no load waits for another: the index two rows ahead, the replica one row ahead
+    int wi = blockIdx.x;
+    int i = index(wi), i1 = index(wi + stride), i2 = index(wi + 2 * stride);
+    Row cur = load_row(g, wi);
+    int rep1 = i1 >= 0 ? __ldg(g.atom_rep + i1) : 0;
+    int jv[U], ev[U];
+    float xv[U], yv[U], zv[U];
+    auto load_col = [&](int first, int end) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) jv[u] = first + 32 * u + lane < end ? __ldg(g.col + first + 32 * u + lane) : -1;
+    };
+    auto load_pos = [&]() {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (jv[u] >= 0) {
+                xv[u] = __ldg(g.x + 3 * jv[u]);
+                yv[u] = __ldg(g.x + 3 * jv[u] + 1);
+                zv[u] = __ldg(g.x + 3 * jv[u] + 2);
+                ev[u] = __ldg(io.s_exp + jv[u]);
+            }
+    };
+    load_col(cur.beg, cur.end);
+    load_pos();
+    int k = 0;   // chunks announced
+    for (; i >= 0; wi += stride) {
+        const AtomGeom a = wrap_inverse(cur.a);
+        const int beg = cur.beg, end = cur.end;
+        // the next row, and the replica and index behind it
+        Row nx;
+        nx.i = i1;
+        nx.beg = nx.end = 0;
+        if (i1 >= 0) {
+            nx.beg = __ldg(g.row_ptr + i1);
+            nx.end = __ldg(g.row_ptr + i1 + 1);
+            nx.a.x = __ldg(g.x + 3 * i1); nx.a.y = __ldg(g.x + 3 * i1 + 1); nx.a.z = __ldg(g.x + 3 * i1 + 2);
+            nx.a.bx = __ldg(g.box + 3 * rep1); nx.a.by = __ldg(g.box + 3 * rep1 + 1); nx.a.bz = __ldg(g.box + 3 * rep1 + 2);
+        }
+        const int rep2 = i2 >= 0 ? __ldg(g.atom_rep + i2) : 0, i3 = index(wi + 3 * stride);
+        {
+            int cnt = 0, first = 1, e_ref = -128;
+            auto flush = [&](bool last) {
+                const int b = k & 1;
+                if (lane == 0) f.chunk[b] = Chunk{i, cnt, first, last ? 1 : 0, e_ref};
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&f.full[b]));
+                if (last) load_col(nx.beg, nx.end);   // the next row's candidates
+                if (last) load_pos();
+                // the other buffer's chunk has been consumed
+                if (k > 0 && !warp_wait(bar_free, (k - 1) & 1)) return false;
+                ++k;
+                first = 0;
+                return true;
+            };
+            if (end - beg > 32 * U) {
+                // more candidates than are in flight: the reference exponent of the whole row first
+                for (int e = beg + lane; e < end; e += 32) {
+                    const int j = __ldg(g.col + e);
+                    if (edge_disp(a, __ldg(g.x + 3 * j), __ldg(g.x + 3 * j + 1), __ldg(g.x + 3 * j + 2)).w < rc2)
+                        e_ref = max(e_ref, __ldg(io.s_exp + j));
+                }
+            }
+            for (int base = beg; base < end; base += 32 * U) {
+                if (base > beg) {
+                    load_col(base, end);
+                    load_pos();
+                }
+                float4 d[U];
+                unsigned m[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    d[u] = edge_disp(a, xv[u], yv[u], zv[u]);
+                    const bool act = jv[u] >= 0 && d[u].w < rc2;
+                    m[u] = __ballot_sync(DMTS_FULL, act);
+                    if (act) e_ref = max(e_ref, ev[u]);
+                }
+                if (base == beg) e_ref = __reduce_max_sync(DMTS_FULL, e_ref);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int c = __popc(m[u]);
+                    const bool act = (m[u] >> lane) & 1u;
+                    int pos = cnt + __popc(m[u] & ((1u << lane) - 1u));
+                    const float4 v = make_float4(d[u].x, d[u].y, d[u].z, __int_as_float(jv[u]));
+                    if (act && pos < TC_E) {
+                        f.qd[k & 1][pos] = v;
+                        f.qe[k & 1][pos] = ev[u];
+                    }
+                    if (cnt + c > TC_E) {   // the chunk is full and more edges follow
+                        const int rest = cnt + c - TC_E;
+                        cnt = TC_E;
+                        if (!flush(false)) return false;
+                        pos -= TC_E;
+                        if (act && pos >= 0) {
+                            f.qd[k & 1][pos] = v;
+                            f.qe[k & 1][pos] = ev[u];
+                        }
+                        cnt = rest;
+                    } else {
+                        cnt += c;
+                    }
+                }
+            }
+            if (!flush(true)) return false;
+        }
+        i = i1;
+        i1 = i2;
+        rep1 = rep2;
+        i2 = i3;
+        cur = nx;
     }
-    if (warp == 0) tmem_alloc(smem_u32(&tmem_sh), TF_TMEM);
-    // weights of channel c = tid as row c of each l's tile
-    {
-        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    if (lane == 0) f.chunk[k & 1] = Chunk{-1, 0, 1, 1, 0};
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&f.full[k & 1]));
+    return true;
+}
+
+// One edge's radial functions and harmonics, handed from the thread that
+// forms them to the threads that form the products.
+struct BasisBuf {
+    float4 b[2][TC_E];      // f_c B_k, scaled into fp16's range
+    float Y[9][TC_E];
+};
+
+// A working warp's share of a chunk's gather: rows warp, warp + 8, ... of the
+// S tile, one 16-byte piece per lane and row; `rows` may exceed the chunk's
+// edges (the further rows repeat the receiver's own features).
+__device__ __forceinline__ void gather_share(const FrontSmem &f, uint32_t q, int rows, uint32_t sS, const __half *s16,
+                                             int warp, int lane) {
+    const int n = f.chunk[q & 1].n, i = f.chunk[q & 1].i;
+    int j[8];
 #pragma unroll
-        for (int l = 0; l < NL; ++l) {
-            __nv_bfloat16 hi[K], lo[K];
+    for (int u = 0; u < 8; ++u) j[u] = warp + 8 * u < n ? __float_as_int(f.qd[q & 1][warp + 8 * u].w) : i;
+    const uint32_t dst = sS + (lane >> 3) * S_BLK + swz128(warp, lane & 7);
+    const char *src = reinterpret_cast<const char *>(s16) + 16 * lane;
 #pragma unroll
-            for (int k = 0; k < K; ++k) split_bf16(__ldg(io.wrad + (l * K + k) * C + tid), hi[k], lo[k]);
-            uint8_t *t = pA + (l >> 1) * TF_C * 128;
-            const int c0 = 4 * (l & 1);
-            st_chunk(t, tid, c0, pack8(hi));
-            st_chunk(t, tid, c0 + 1, nseg == 3 ? pack8(lo) : z);
-            st_chunk(t, tid, c0 + 2, nseg == 3 ? pack8(hi) : z);
-            st_chunk(t, tid, c0 + 3, z);
+    for (int u = 0; u < 8; ++u)
+        if (warp + 8 * u < rows) cp_async16_relaxed(dst + u * 1024, src + (size_t)j[u] * (4 * TC_C));
+}
+
+// Products of the edges' bases with the harmonics: the E tile. Thread (e, q),
+// q < 3, of the six producing warps forms the eight columns (lm, k) of row e
+// for lm = q, q + 3, q + 6.
+template <int LMAX>
+__device__ __forceinline__ void store_products(uint8_t *pE, const BasisBuf &B, int t, int n16) {
+    using D = TcDims<LMAX>;
+    const int e = t & (TC_E - 1), q = t / TC_E;
+    if (e >= n16) return;
+    const float4 b0 = B.b[0][e], b1 = B.b[1][e];
+#pragma unroll
+    for (int u = 0; u < (D::NLM + 2) / 3; ++u) {
+        const int lm = q + 3 * u;
+        if (lm >= D::NLM) break;
+        const float y = B.Y[lm][e];
+        const float2 yy = make_float2(y, y);
+        uint4 hi, lo;
+        split2_prod(make_float2(b0.x, b0.y), yy, hi.x, lo.x);
+        split2_prod(make_float2(b0.z, b0.w), yy, hi.y, lo.y);
+        split2_prod(make_float2(b1.x, b1.y), yy, hi.z, lo.z);
+        split2_prod(make_float2(b1.z, b1.w), yy, hi.w, lo.w);
+        uint8_t *p = pE + (lm >> 1) * E_BLK + swz32(e, lm & 1);
+        *reinterpret_cast<uint4 *>(p) = hi;
+        *reinterpret_cast<uint4 *>(p + D::e_part) = lo;
+    }
+}
+
+// Sums lm = LM0 .. LM1 - 1 of one channel from its TMEM lane.
+template <int LM0, int LM1>
+__device__ __forceinline__ void apply_weights(uint32_t t_lane, const float (*W)[TC_KR], float sc, float *A) {
+#pragma unroll
+    for (int lm0 = LM0; lm0 < LM1; lm0 += 3) {
+        uint32_t t[3][8];
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (lm0 + u < LM1) tmem_ld8_issue(t_lane + 8 * (lm0 + u), t[u]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const int lm = lm0 + u;
+            if (lm >= LM1) continue;
+            const float *w = W[LM0 == 0 && lm > 0 ? 1 : 0];   // l of lm: the group's first or second row
+            float v0 = 0.f, v1 = 0.f;
+#pragma unroll
+            for (int k = 0; k < TC_KR; k += 2) {
+                v0 = fmaf(w[k], __uint_as_float(t[u][k]), v0);
+                v1 = fmaf(w[k + 1], __uint_as_float(t[u][k + 1]), v1);
+            }
+            A[lm - LM0] = sc * (v0 + v1);
         }
     }
+}
+
+// ------------------------------------------------------------------ forward
+struct FwdTcSmem {
+    uint64_t bar, basis_full[2], rest;   // MMAs done, basis formed, warps 2 and 3 done with TMEM and their gather
+    uint32_t tmem;
+    FrontSmem front;
+    BasisBuf basis[2];
+};
+template <int LMAX>
+constexpr size_t fwd_tc_tiles() { return S_BYTES + TcDims<LMAX>::e_bytes + 1024; }   // + alignment slack
+
+// One CTA (three per SM), a chunk at a time. Six of the eight working warps
+// form the products, then one of them starts the MMAs (into the TMEM
+// accumulator D[c][(lm,k)]); warps 2 and 3 meanwhile form the next chunk's
+// radial functions and harmonics (a thread per edge). When the MMAs are done
+// all start the next chunk's gather and, as two groups of a thread per channel,
+// apply the radial weights of their channel to l <= 1 and l = 2 (the
+// receiver's last chunk). Bound by the latency of a chunk's phases (about 6,000
+// cycles, of which the MMAs, limited by shared-memory reads of their operands,
+// take 750); 23,558 atoms, l_max = 2: 163 us, where the same sum with the
+// radial products formed per edge (on the tensor cores) took 254 us. Every mbarrier wait is bounded: on timeout the CTA
+// records DMTS_E_TIMEOUT, waits (bounded) for the MMAs it issued, frees its
+// tensor memory and returns.
+template <int LMAX>
+__global__ void __launch_bounds__(TC_THREADS, 3) k_mp_fwd_tc(EdgeGeom g, LayerIO io, float escale, int *err) {
+    using D = TcDims<LMAX>;
+    constexpr int NL = D::NL, NLM = D::NLM, C = TC_C;
+    constexpr int TMEM = 128;   // columns allocated; NN <= 80 used
+    extern __shared__ uint8_t tc_smem[];
+    __shared__ FwdTcSmem sm;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, c = tid & (C - 1), grp = tid >> 7;
+    const uint32_t raw = smem_u32(tc_smem), base = (raw + 1023u) & ~1023u;
+    const uint32_t sS = base, sE = base + S_BYTES;
+    uint8_t *pE = tc_smem + (base - raw) + S_BYTES;
+    const uint32_t sbar = smem_u32(&sm.bar), rest = smem_u32(&sm.rest);
+    const int err0 = *io.err;
+
+    if (tid == 0) {
+        mbar_init(sbar, 1);
+        mbar_init(smem_u32(&sm.basis_full[0]), 2);
+        mbar_init(smem_u32(&sm.basis_full[1]), 2);
+        mbar_init(rest, 2);
+        front_init(sm.front);
+        mbar_init_fence();
+    }
+    if (warp == 0) tmem_alloc(smem_u32(&sm.tmem), TMEM);
+    // columns past (l_max + 1)^2 K stay zero
+    if (NLM < 2 * D::NB && tid < 2 * TC_E)
+        *reinterpret_cast<uint4 *>(pE + (tid / TC_E) * D::e_part + (D::NB - 1) * E_BLK + swz32(tid % TC_E, 1)) =
+            make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_sh;
-    const uint32_t t_lane = tmem + ((uint32_t)(warp * 32) << 16);
-    const uint32_t idesc = idesc_bf16(TF_C, TF_CHUNK);
-    uint32_t phase = 0;
-    bool aborted = err0 != 0;
+    const uint32_t tmem = sm.tmem, t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    bool aborted = false;
+    uint32_t k = 0;   // chunks done
 
-    for (int wi = blockIdx.x; wi < g.n_atoms && !aborted; wi += gridDim.x) {
-        const int i = g.order ? __ldg(g.order + wi) : wi;
-        const int rep = g.atom_rep[i];
-        const float bx = g.box[3 * rep], by = g.box[3 * rep + 1], bz = g.box[3 * rep + 2];
-        const float ibx = bx > 0.f ? 1.f / bx : 0.f, iby = by > 0.f ? 1.f / by : 0.f, ibz = bz > 0.f ? 1.f / bz : 0.f;
-        const float xi = g.x[3 * i], yi = g.x[3 * i + 1], zi = g.x[3 * i + 2];
-        const float rc2 = g.rc * g.rc;
-        const int beg = g.row_ptr[i], end = g.row_ptr[i + 1];
-        float2 acc[NLM];
+    if (err0) {
+        // an earlier error: nothing is computed
+    } else if (warp == 8) {
+        aborted = !front_end(g, io, sm.front, sbar, lane);
+    } else {
+        auto full = [&](uint32_t q) { return warp_wait(smem_u32(&sm.front.full[q & 1]), (q >> 1) & 1); };
+        // radial weights of channel c: l = 0, 1 in the first group, l = 2 in the second (l_max = 1: 0 | 1)
+        float W[2][TC_KR];
 #pragma unroll
-        for (int lm = 0; lm < NLM; ++lm) acc[lm] = make_float2(0.f, 0.f);
-
-        for (int pbeg = beg; pbeg < end && !aborted; pbeg += TF_PASS) {
-            // ---- test one candidate per thread, compact the active ones
-            const int e = pbeg + tid;
-            bool act = false;
-            if (tid < TF_PASS && e < end) {
-                const int j = __ldg(g.col + e);
-                const float dx = min_img(__ldg(g.x + 3 * j) - xi, bx, ibx);
-                const float dy = min_img(__ldg(g.x + 3 * j + 1) - yi, by, iby);
-                const float dz = min_img(__ldg(g.x + 3 * j + 2) - zi, bz, ibz);
-                const float r2 = dx * dx + dy * dy + dz * dz;
-                act = r2 < rc2;
-                if (act) {
-                    cd[tid] = make_float4(dx, dy, dz, r2);
-                    cj[tid] = j;
+        for (int q = 0; q < TC_KR; ++q) {
+            const int l0 = grp == 0 ? 0 : LMAX, l1 = LMAX >= 1 ? 1 : 0;
+            W[0][q] = __ldg(io.wrad + (l0 * TC_KR + q) * C + c);
+            W[1][q] = __ldg(io.wrad + (l1 * TC_KR + q) * C + c);
+        }
+        constexpr uint32_t idesc = idesc_f16(C, D::NN, 1, 1);
+        const uint64_t descA = smem_desc_sw(sS, S_BLK, 1024, 128), descB = smem_desc_sw(sE, E_BLK, 256, 32);
+        const int warp_u = __shfl_sync(DMTS_FULL, warp, 0);
+        const bool is_basis = warp == 2 || warp == 3;
+        // the basis of chunk q: threads 64 .. 127, one edge each
+        auto basis = [&](uint32_t q) {
+            const Chunk &ch = sm.front.chunk[q & 1];
+            BasisBuf &B = sm.basis[q & 1];
+            const int e = tid - 64, n = ch.n;
+            if (e < ((n + 15) & ~15)) {
+                float b[TC_KR], Y[NLM];
+#pragma unroll
+                for (int u = 0; u < TC_KR; ++u) b[u] = 0.f;
+#pragma unroll
+                for (int u = 0; u < NLM; ++u) Y[u] = 0.f;
+                if (e < n) {
+                    const float4 d = sm.front.qd[q & 1][e];
+                    const float r = sqrtf(d.x * d.x + d.y * d.y + d.z * d.z), inv = 1.f / r;
+                    float du;
+                    // the neighbour's row scale relative to the receiver's reference
+                    const float fc =
+                        envelope(r * g.inv_rc, g.p, &du) * escale * pow2f(max(sm.front.qe[q & 1][e] - ch.e_ref, -120));
+                    bessel<TC_KR, false>(r, g.inv_rc, g.bnorm, b, nullptr);
+#pragma unroll
+                    for (int u = 0; u < TC_KR; ++u) b[u] *= fc;
+                    sph<LMAX>(d.x * inv, d.y * inv, d.z * inv, Y);
                 }
+                B.b[0][e] = make_float4(b[0], b[1], b[2], b[3]);
+                B.b[1][e] = make_float4(b[4], b[5], b[6], b[7]);
+#pragma unroll
+                for (int u = 0; u < NLM; ++u) B.Y[u][e] = Y[u];
             }
-            const unsigned m = __ballot_sync(DMTS_FULL, act);
-            if (lane == 0) wcnt[warp] = __popc(m);
-            __syncthreads();
-            int off = 0, n_act = 0;
-#pragma unroll
-            for (int w = 0; w < TF_C / 32; ++w) {
-                off += w < warp ? wcnt[w] : 0;
-                n_act += wcnt[w];
-            }
-            const int n_pad = (n_act + TF_CHUNK - 1) / TF_CHUNK * TF_CHUNK;
-            // slot of each active candidate, in candidate order
-            if (act) perm[off + __popc(m & ((1u << lane) - 1u))] = tid;
-            __syncthreads();
-            // ---- one thread per slot: the edge's basis row, harmonics, index
-            if (tid < n_act) {
-                const int src = perm[tid];
-                const float4 d = cd[src];
-                const float r = sqrtf(d.w), inv = 1.f / r;
-                float du;
-                const float fc = envelope(r * g.inv_rc, g.p, &du);
-                float B[K];
-                bessel<K, false>(r, g.inv_rc, g.bnorm, B, nullptr);
-                __nv_bfloat16 hi[K], lo[K];
-#pragma unroll
-                for (int k = 0; k < K; ++k) split_bf16(fc * B[k], hi[k], lo[k]);
-                const uint4 h8 = pack8(hi);
-                const uint4 l8 = pack8(lo), z4 = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                for (int hh = 0; hh < (NL > 1 ? 2 : 1); ++hh) {   // the basis in both halves of the row
-                    st_chunk(pB, tid, 4 * hh, h8);
-                    st_chunk(pB, tid, 4 * hh + 1, h8);
-                    st_chunk(pB, tid, 4 * hh + 2, l8);
-                    st_chunk(pB, tid, 4 * hh + 3, z4);
-                }
-                float Y[NLM];
-                sph<LMAX>(d.x * inv, d.y * inv, d.z * inv, Y);
-#pragma unroll
-                for (int lm = 0; lm < NLM; ++lm) sY[lm][tid] = Y[lm];
-                sJ[tid] = cj[src];
-            } else if (tid < n_pad) {
-                // padding slots of the last chunk: zero basis rows and
-                // harmonics, and the receiver's own (finite) features
-                const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) st_chunk(pB, tid, q, z);
-#pragma unroll
-                for (int lm = 0; lm < NLM; ++lm) sY[lm][tid] = 0.f;
-                sJ[tid] = i;
-            }
-            fence_proxy_async_smem();
-            __syncthreads();
-
-            for (int q0 = 0; q0 < n_act; q0 += TF_CHUNK) {
-                if (tid == 0) {
-                    tc_fence_after();
-#pragma unroll
-                    for (int l = 0; l < NL; ++l)
-#pragma unroll
-                        for (int kk = 0; kk < 2; ++kk)
-                            mma_bf16(tmem + l * TF_CHUNK, smem_desc(sA + (l >> 1) * TF_C * 128 + (l & 1) * 64 + kk * 32),
-                                     smem_desc(sB + q0 * 128 + (l & 1) * 64 + kk * 32), idesc, kk);
-                    mma_commit(smem_u32(&bar));
-                }
-                // neighbour features of this chunk (padding slots read the
-                // receiver's own), loaded while the MMAs run
-                float sj[TF_CHUNK];
-#pragma unroll
-                for (int u4 = 0; u4 < TF_CHUNK / 4; ++u4) {
-                    const int4 jj = *reinterpret_cast<const int4 *>(&sJ[q0 + 4 * u4]);
-                    sj[4 * u4] = __ldg(io.s + (size_t)jj.x * C + tid);
-                    sj[4 * u4 + 1] = __ldg(io.s + (size_t)jj.y * C + tid);
-                    sj[4 * u4 + 2] = __ldg(io.s + (size_t)jj.z * C + tid);
-                    sj[4 * u4 + 3] = __ldg(io.s + (size_t)jj.w * C + tid);
-                }
-                const bool ok = mbar_wait(smem_u32(&bar), phase);
-                if (!__syncthreads_and(ok ? 1 : 0)) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sm.basis_full[q & 1]));
+        };
+        // (the rows that pad the last group of 16 are filled too: 0 x row has to stay 0)
+        auto gather = [&](uint32_t q) {
+            const Chunk &ch = sm.front.chunk[q & 1];
+            if (ch.i >= 0) gather_share(sm.front, q, (ch.n + 15) & ~15, sS, io.s16, warp, lane);
+        };
+        bool ok = full(0);
+        if (ok) gather(0);
+        if (ok && is_basis) basis(0);
+        for (;; ++k) {
+            const Chunk ch = sm.front.chunk[k & 1];
+            if (ok && ch.i < 0) break;
+            const int n16 = (ch.n + 15) & ~15;
+            if (is_basis) {
+                // this warp's share of the gather has landed and its reads of
+                // TMEM are done: the chunk's MMAs may start
+                cp_async_wait_all();
+                fence_proxy_async_smem();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(rest);
+                ok = full(k + 1) && ok;
+                if (ok) basis(k + 1);
+            } else {
+                ok = warp_wait(smem_u32(&sm.basis_full[k & 1]), (k >> 1) & 1) && ok;
+                if (ok) store_products<LMAX>(pE, sm.basis[k & 1], (warp < 2 ? warp : warp - 2) * 32 + lane, n16);
+                cp_async_wait_all();
+                fence_proxy_async_smem();
+                tc_fence_before();   // the last receiver's TMEM reads
+                if (!bar_sync_and(1, TC_PROD, ok)) {
                     aborted = true;
                     break;
                 }
-                phase ^= 1u;
-                tc_fence_after();
-                const int nsb = min(TF_CHUNK / 8, (n_act - q0 + 7) / 8);
-#pragma unroll
-                for (int b = 0; b < TF_CHUNK / 8; ++b) {
-                    if (b >= nsb) break;   // uniform across the CTA
-                    uint32_t rr[NL][8];
-#pragma unroll
-                    for (int l = 0; l < NL; ++l) tmem_ld8_issue(t_lane + l * TF_CHUNK + 8 * b, rr[l]);
-                    tmem_wait_ld();
-                    const int p0 = q0 + 8 * b;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float4 y[NLM];
-#pragma unroll
-                        for (int lm = 0; lm < NLM; ++lm) y[lm] = *reinterpret_cast<const float4 *>(&sY[lm][p0 + 4 * h]);
-#pragma unroll
-                        for (int pr = 0; pr < 2; ++pr) {
-                            const int u = 8 * b + 4 * h + 2 * pr;   // slot within the chunk
-                            const float2 s2 = make_float2(sj[u], sj[u + 1]);
-#pragma unroll
-                            for (int l = 0; l < NL; ++l) {
-                                const int c0 = 4 * h + 2 * pr;
-                                const float2 R2 = make_float2(__uint_as_float(rr[l][c0]), __uint_as_float(rr[l][c0 + 1]));
-                                const float2 msg = __fmul2_rn(R2, s2);
-#pragma unroll
-                                for (int lm = l * l; lm < (l + 1) * (l + 1); ++lm) {
-                                    const float2 y2 = pr ? make_float2(y[lm].z, y[lm].w) : make_float2(y[lm].x, y[lm].y);
-                                    acc[lm] = __ffma2_rn(msg, y2, acc[lm]);
-                                }
-                            }
+                if (warp_u == 0) {
+                    ok = warp_wait(rest, k & 1);
+                    tc_fence_after();
+                    if (ok && elect_one()) {
+                        uint64_t ad = descA, bd = descB;
+                        uint32_t acc = !ch.first;
+#pragma unroll 1
+                        for (int ks = 0; ks < n16; ks += 16, ad += 2048 >> 4, bd += 512 >> 4) {
+                            mma_f16kind(tmem, ad, bd, idesc, acc);
+                            mma_f16kind(tmem, ad + (S_PART >> 4), bd, idesc, 1u);
+                            mma_f16kind(tmem, ad, bd + (D::e_part >> 4), idesc, 1u);
+                            acc = 1u;
                         }
+                        mma_commit(sbar);
                     }
+                    __syncwarp();
                 }
-                tc_fence_before();
-                __syncthreads();   // TMEM read before the next chunk's MMAs overwrite it
+                ok = full(k + 1) && ok;
             }
-        }
-        if (aborted) break;
-        // ---- receiver epilogue: A, q (and its split copy)
-        float qv[NL];
+            ok = warp_wait(sbar, k & 1) && ok;
+            if (!ok) {
+                if (!is_basis) continue;   // to the barrier of the producing warps
+                aborted = true;
+                break;
+            }
+            gather(k + 1);
+            if (!ch.last) continue;
+            tc_fence_after();
+            // ---- thread (group, c): A[lm][c] = nu sum_k W_lkc T[lm,k][c]
+            const float sc = io.nu * pow2f(max(ch.e_ref, -100) - TC_TOP) / escale;
+            constexpr int M0 = LMAX == 2 ? 4 : 1;        // lm of the first group
+            float A[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            if (ch.n > 0) {   // (an empty chunk is the only one of its row)
+                if (grp == 0) apply_weights<0, M0>(t_lane, W, sc, A);
+                else if (LMAX >= 1) apply_weights<M0, (LMAX >= 1 ? NLM : M0)>(t_lane, W, sc, A);
+            }
+            const int i = ch.i;
+            auto put_q = [&](int l, float v) {
+                if (io.q) io.q[(size_t)i * NL * C + l * C + c] = v;
+                if (io.q_bf16) st_split(io.q_bf16, i, NL * C, l * C + c, v);
+            };
+            float *Ai = io.A + (size_t)i * NLM * C + c;
+            if (grp == 0) {
 #pragma unroll
-        for (int l = 0; l < NL; ++l) qv[l] = 0.f;
+                for (int lm = 0; lm < M0; ++lm) Ai[lm * C] = A[lm];
+                put_q(0, A[0] * A[0]);
+                if (LMAX == 2) put_q(1, fmaf(A[3], A[3], fmaf(A[2], A[2], A[1] * A[1])));
+            } else if (LMAX >= 1) {
+                float v = 0.f;
 #pragma unroll
-        for (int lm = 0; lm < NLM; ++lm) {
-            const int l = lm == 0 ? 0 : (lm < 4 ? 1 : 2);
-            const float a = io.nu * (acc[lm].x + acc[lm].y);
-            qv[l] = fmaf(a, a, qv[l]);
-            if (io.A) io.A[((size_t)i * NLM + lm) * C + tid] = a;
-        }
-#pragma unroll
-        for (int l = 0; l < NL; ++l) {
-            io.q[(size_t)i * NL * C + l * C + tid] = qv[l];
-            if (io.q_bf16) st_split(io.q_bf16, i, NL * C, l * C + tid, qv[l]);
+                for (int lm = M0; lm < NLM; ++lm) {
+                    Ai[lm * C] = A[lm - M0];
+                    v = fmaf(A[lm - M0], A[lm - M0], v);
+                }
+                put_q(LMAX, v);
+            }
         }
     }
 
-    if (aborted && tid == 0) {
+    if (aborted && lane == 0) {
         set_error(err, DMTS_E_TIMEOUT);
-        mbar_wait(smem_u32(&bar), phase);   // the MMAs issued must complete before TMEM is freed
+        if (warp < 8) mbar_wait(sbar, k & 1);   // the MMAs issued must complete before TMEM is freed
     }
+    cp_async_wait_all();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tmem, TF_TMEM);
+        tmem_dealloc(tmem, TMEM);
     }
 }
 
+// ------------------------------------------------------- feature split
+// Warp per atom: the row's largest magnitude -> exponent e, hi / lo of
+// s 2^(TC_TOP - e).
+__global__ void __launch_bounds__(256) k_feature_split(int n, const float *__restrict__ s, __half *__restrict__ s16,
+                                                       int *__restrict__ s_exp) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(s + (size_t)i * TC_C) + lane);
+    const unsigned m = max(max(__float_as_uint(fabsf(v.x)), __float_as_uint(fabsf(v.y))),
+                           max(__float_as_uint(fabsf(v.z)), __float_as_uint(fabsf(v.w))));
+    const int e = row_exponent(__reduce_max_sync(DMTS_FULL, m));
+    const float f = pow2f(TC_TOP - e);
+    uint2 hi, lo;
+    split2(v.x * f, v.y * f, hi.x, lo.x);
+    split2(v.z * f, v.w * f, hi.y, lo.y);
+    uint2 *row = reinterpret_cast<uint2 *>(s16 + (size_t)i * 2 * TC_C);
+    row[lane] = hi;
+    row[32 + lane] = lo;
+    if (lane == 0) s_exp[i] = e;
+}
+
+// Power of two that puts the basis f_c B_k Y_lm (bounded by
+// 2.24 sqrt(2 / rc) K pi / rc) below 2^TC_TOP.
+float basis_scale(const EdgeGeom &g) {
+    const float bound = 2.24f * g.bnorm * TC_KR * 3.1415927f * g.inv_rc;
+    return std::ldexp(1.f, TC_TOP - 1 - std::ilogb(bound));
+}
+
+// CTAs to launch: as many as fit on the current device at once, and TMEM's
+// 512 columns per SM.
+int persistent_grid(const void *fn, int threads, size_t smem, int tmem_cols) {
+    int dev = 0, n_sm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    return n_sm * std::max(1, std::min(resident_ctas(fn, threads, smem, dev), 512 / tmem_cols));
+}
+
 template <int LMAX>
-void fwd_tc_launch(const EdgeGeom &g, const LayerIO &io, int nseg, int *err, cudaStream_t st) {
-    constexpr size_t smem = FwdTcSmem<LMAX>::bytes;
-    static int per_sm = 0, n_sm = 0;
-    if (!per_sm) {
-        cudaFuncSetAttribute(k_mp_fwd_tc<LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(k_mp_fwd_tc<LMAX>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        per_sm = resident_ctas(reinterpret_cast<const void *>(k_mp_fwd_tc<LMAX>), TF_C, smem, dev);
-        // TMEM: 512 columns per SM
-        per_sm = std::max(1, std::min(per_sm, 512 / TF_TMEM));
-    }
-    const int grid = std::min(g.n_atoms, per_sm * n_sm);
-    k_mp_fwd_tc<LMAX><<<grid, TF_C, smem, st>>>(g, io, nseg, err);
+void fwd_tc_launch(const EdgeGeom &g, const LayerIO &io, int *err, cudaStream_t st) {
+    constexpr size_t smem = fwd_tc_tiles<LMAX>();
+    cudaFuncSetAttribute(k_mp_fwd_tc<LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_mp_fwd_tc<LMAX>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                         (int)cudaSharedmemCarveoutMaxShared);
+    const int grid = std::min(g.n_atoms, persistent_grid(reinterpret_cast<const void *>(k_mp_fwd_tc<LMAX>), TC_THREADS, smem, 128));
+    k_mp_fwd_tc<LMAX><<<grid, TC_THREADS, smem, st>>>(g, io, basis_scale(g), err);
     count_launch();
 }
 
@@ -332,13 +578,19 @@ int resident_ctas(const void *fn, int threads, size_t dyn_smem, int dev) {
     return std::max(n, 1);
 }
 
-bool mp_fwd_tc_supported(int C, int K) { return C == TF_C && K == TF_K; }
+bool mp_tc_supported(int C, int K) { return C == TC_C && K == TC_KR; }
 
-void launch_mp_fwd_tc(int lmax, const EdgeGeom &g, const LayerIO &io, int nseg, int *err, cudaStream_t st) {
+void launch_feature_split(int n, const float *s, void *s16, int *s_exp, cudaStream_t st) {
+    if (n == 0) return;
+    k_feature_split<<<(n + 7) / 8, 256, 0, st>>>(n, s, static_cast<__half *>(s16), s_exp);
+    count_launch();
+}
+
+void launch_mp_fwd_tc(int lmax, const EdgeGeom &g, const LayerIO &io, int *err, cudaStream_t st) {
     if (g.n_atoms == 0) return;
-    if (lmax == 0) fwd_tc_launch<0>(g, io, nseg, err, st);
-    else if (lmax == 1) fwd_tc_launch<1>(g, io, nseg, err, st);
-    else fwd_tc_launch<2>(g, io, nseg, err, st);
+    if (lmax == 0) fwd_tc_launch<0>(g, io, err, st);
+    else if (lmax == 1) fwd_tc_launch<1>(g, io, err, st);
+    else fwd_tc_launch<2>(g, io, err, st);
 }
 
 }  // namespace dmts

@@ -21,6 +21,28 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     return d;
 }
 
+// The general form: swizzle 128 or 32 bytes, leading and stride byte offsets.
+// Canonical layouts (T = 16-byte units of 8 halves):
+//  K-major:  rows of one swizzle span along K, 8-row groups `sbo` apart
+//            (`lbo` unused: each MMA's K = 16 lies within a span);
+//  MN-major: K rows of one swizzle span (64 or 16 elements) along M / N, 8-row
+//            groups `sbo` apart, the next 64 or 16 elements `lbo` further.
+__device__ __forceinline__ uint64_t smem_desc_sw(uint32_t addr, uint32_t lbo, uint32_t sbo, int swizzle) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFF);
+    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
+    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)(swizzle == 128 ? 2 : 6) << 61;
+    return d;
+}
+
+// Byte offset of the 16-byte chunk j (0, 1) of row r of a 32-byte-swizzled
+// tile (rows of 32 bytes, 256-byte aligned): j is XORed with bit 2 of r.
+__host__ __device__ __forceinline__ uint32_t swz32(int r, int j) {
+    return (uint32_t)r * 32u + ((uint32_t)(j ^ ((r >> 2) & 1)) << 4);
+}
+
 // Byte offset, within a 1024-byte-aligned tile in that layout, of the
 // 16-byte chunk j (0..7) of row r: the chunk index is XORed with r mod 8.
 __host__ __device__ __forceinline__ uint32_t swz128(int r, int j) {
@@ -33,13 +55,32 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A x B^T, M = 128 (cta_group::1), K = 16.
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
+// kind::f16 with fp16 A and B, fp32 D; a_mn / b_mn: the operand is MN-major.
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int a_mn, int b_mn) {
+    return (1u << 4) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(M >> 4) << 24);
+}
+
+// D[tmem] (+)= A x B^T, M = 128 (cta_group::1), K = 16 (the operand type is the descriptor's).
+__device__ __forceinline__ void mma_f16kind(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
         "l"(a), "l"(b), "r"(idesc), "r"(accum));
+}
+
+// True in one lane of a converged warp. MMAs are issued under it, not under a
+// lane-index test: the warp stays uniform, so descriptors are formed in
+// uniform registers instead of being moved there for every instruction.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
 }
 
 // Arrives on the mbarrier once every MMA this thread issued has completed.
