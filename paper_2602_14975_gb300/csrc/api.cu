@@ -495,6 +495,7 @@ dmts_status nc_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const i
     if (!(flags & kFlagEmbedded)) { ProfScope ps(ctx, "embed", st); launch_embed(N, C, s.species, m.emb, s0, st); }
     FirstIO io = first_io(ctx, s, m);
     io.A = (flags & kFlagKeepPre) ? (float *)w.dist_A.p : nullptr;   // the head needs q and V only; kept for the distillation
+    io.T = (flags & kFlagKeepPre) ? (float *)w.dist_T.p : nullptr;
     // the tensor-core path reads only the split-bf16 copy; the distillation's
     // weight gradient reads the fp32 one
     io.q = (bf && !(flags & kFlagKeepPre)) ? nullptr : (float *)w.nc_q.p;
@@ -1050,15 +1051,16 @@ dmts_status nc_distill_step(dmts_ctx *ctx, const dmts_system *sys, const dmts_nb
     Workspace &w = ctx->ws;
     const int N = v.n, H = m.K + m.nl, QKW = 2 * H * m.nc, C = m.C;
     const bool fit_mlp = params & DMTS_FIT_MLP, fit_qk = params & DMTS_FIT_QK, fit_layer = params & DMTS_FIT_LAYER;
-    const size_t nb = m.n_weights, part = std::max((size_t)64 * QKW * (C + 1) + (size_t)64 * C * (2 * C + 1),
-                                                   (size_t)1024 * 2 * m.K * C);
+    const size_t nb = m.n_weights, part = std::max((size_t)ATB_SLICES * std::max(QKW * (C + 1), C * (2 * C + 1)),
+                                                   (size_t)WG_BLOCKS * (2 * m.K + m.nl) * C);
     if (!w.dist_F.ensure(sizeof(float) * 3 * (N + 1)) || !w.dist_g.ensure(sizeof(float) * 3 * (N + 1)) ||
         !w.dist_sq.ensure(sizeof(float) * (N + 1)) || !w.dist_gqk.ensure(sizeof(float) * ((size_t)QKW * N + 1)) ||
         !w.dist_gs1.ensure(sizeof(float) * ((size_t)C * N + 1)) || !w.dist_gh.ensure(sizeof(float) * ((size_t)C * N + 1)) ||
         !w.dist_h.ensure(sizeof(float) * ((size_t)C * N + 1)) || !w.dist_dw.ensure(sizeof(float) * nb) ||
         !w.adam_m.ensure(sizeof(float) * nb) || !w.adam_v.ensure(sizeof(float) * nb) ||
         !w.dist_part.ensure(sizeof(float) * part) || !w.ms_scratch.ensure(mean_sub_scratch_bytes(N, v.n_rep)) ||
-        !w.dist_A.ensure(sizeof(float) * ((size_t)4 * C * N + 1)) || !w.dist_gq.ensure(sizeof(float) * ((size_t)2 * C * N + 1)) ||
+        !w.dist_A.ensure(sizeof(float) * ((size_t)4 * C * N + 1)) ||
+        !w.dist_T.ensure(sizeof(float) * ((size_t)m.S * 4 * m.K * N + 1)) || !w.dist_gq.ensure(sizeof(float) * ((size_t)2 * C * N + 1)) ||
         !w.dist_gv.ensure(sizeof(float) * ((size_t)3 * m.nl * N + 1)))
         return fail(ctx, DMTS_E_OOM, "workspace allocation failed");
     // forward: the fast force (it leaves q, the MLP's activations and
@@ -1116,27 +1118,19 @@ dmts_status nc_distill_step(dmts_ctx *ctx, const dmts_system *sys, const dmts_nb
         Epi e = epi(EPI_STORE);
         e.out = (float *)w.dist_gq.p;
         launch_gemm_f32(N, 2 * C, C, gh, m.w1[0], 0, e, st);                           // g_q = g_h W1
-        launch_nc_dU(N, C, m.nl, (const float *)w.dist_gv.p, (const float *)w.dist_A.p, part_buf, at(m.U), st);
         NCLayerGradArgs la;
-        la.x = v.x;
-        la.atom_rep = v.atom_rep;
-        la.box = v.box;
-        la.row_ptr = nbr->row_ptr;
-        la.col = nbr->col;
         la.n_atoms = N;
-        la.rc = m.rc;
-        la.inv_rc = 1.f / m.rc;
-        la.bnorm = sqrtf(2.f / m.rc);
         la.nu = m.nu;
-        la.p = m.p;
-        la.s0 = (const float *)w.nc_s.p;
+        la.emb = m.emb;
+        la.n_species = m.S;
+        la.T = (const float *)w.dist_T.p;
         la.A = (const float *)w.dist_A.p;
         la.gq = (const float *)w.dist_gq.p;
         la.gV = (const float *)w.dist_gv.p;
         la.U = m.U;
         la.n_l = m.nl;
         la.err = ctx->d_err;
-        launch_nc_layer_wgrad(C, la, part_buf, at(m.wrad[0]), st);
+        launch_nc_layer_wgrad(C, la, part_buf, at(m.wrad[0]), at(m.U), st);
     }
     if (lr > 0.f && params) {
         if (adam_step == 1 && (!ck(ctx, cudaMemsetAsync(w.adam_m.p, 0, sizeof(float) * nb, st), "adam reset") ||

@@ -75,14 +75,14 @@ struct Workspace {
     // distillation of the NC model: residual, q/k-row and feature gradients,
     // pre-activation, blob-shaped weight gradient, Adam moments, split sums
     Buf dist_F, dist_g, dist_sq, dist_gqk, dist_gs1, dist_gh, dist_h, dist_dw, adam_m, adam_v, dist_part;
-    Buf dist_A, dist_gq, dist_gv;
+    Buf dist_A, dist_T, dist_gq, dist_gv;
     void release_all() {
         Buf *all[] = {&s, &A, &q, &h, &act, &u, &gz, &gs0, &gs1, &gA, &e_atom, &ftmp, &atom_rep,
                       &nc_s, &nc_q, &nc_act, &nc_qk, &nc_v, &nc_f, &nc_ffix, &nc_next, &nc_sum, &s16, &s_exp,
                       &q_bf, &act_bf, &s_bf, &gz_bf, &gs0_bf, &gs1_bf, &nc_q_bf, &nc_act_bf, &nc_s_bf,
                       &ms_scratch, &nc_w, &cons_w, &cons_ffix, &cons_wfix, &nc_w_last,
                       &dist_F, &dist_g, &dist_sq, &dist_gqk, &dist_gs1, &dist_gh, &dist_h, &dist_dw,
-                      &adam_m, &adam_v, &dist_part, &dist_A, &dist_gq, &dist_gv};
+                      &adam_m, &adam_v, &dist_part, &dist_A, &dist_T, &dist_gq, &dist_gv};
         for (Buf *b : all) b->release();
     }
 };

@@ -203,6 +203,8 @@ __global__ void __launch_bounds__((FirstFwdSmem<C, LMAX>::WARPS * 32), (FirstFwd
         });
         __syncwarp();
         nx = load_row(g, wi + stride);
+        if (io.T)
+            for (int q = lane; q < S * NLM * FL_K; q += 32) io.T[(size_t)i * S * NLM * FL_K + q] = sT[2 * q];
         // ---- channel sums
 #pragma unroll 1
         for (int c0 = lane * CPW; c0 < C; c0 += CP) {

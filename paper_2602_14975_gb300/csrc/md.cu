@@ -1,10 +1,8 @@
 // NC direct-force head (Sec. 2 "Model architecture"), the bonded + LJ prior,
 // and the fused BAOAB/RESPA integrator with Philox4x32-10 noise (Algorithm 1);
 // the replica-local mean subtraction of the fast force; the virial estimator
-// and the piston kernels of the NPT path (Sec. 2, virial term in NPT); and
-// the adjoint of the fast force with respect to its weights (head, weight
-// contractions, layer gradients) with the Adam update, for distillation of
-// the NC model (Sec. 2, "Model training").
+// and the piston kernels of the NPT path (Sec. 2, virial term in NPT). The
+// adjoint of the fast force with respect to its weights: distill.cu.
 #include <algorithm>
 #include "md.cuh"
 #include "mp.cuh"
@@ -569,357 +567,6 @@ void launch_nc_head(int K, int n_c, int n_l, const NCHeadArgs &a, cudaStream_t s
     else if (K == 8 && n_c == 8 && n_l == 1) nc_head_launch<8, 8, 1>(a, st);
     else if (K == 8 && n_c == 8 && n_l == 3) nc_head_launch<8, 8, 3>(a, st);
     else if (K == 8 && n_c == 8 && n_l == 4) nc_head_launch<8, 8, 4>(a, st);
-}
-
-// ------------------------------------------------- NC head adjoint (q/k)
-// Warp per atom a. Lane h < H owns head h of c_ajh = q_ah . k_jh / sqrt(n_c)
-// (and accumulates dL/dq_ah), lane H + h owns c_jah = q_jh . k_ah / sqrt(n_c)
-// (dL/dk_ah). With F_aj = f_c S_aj (n + T_aj), S_aj = sum_{h<K} c_ajh B_h,
-// T_aj = sum_t c_aj(K+t) V_at, F_ja = f_c S_ja (-n + T_ja) and
-// F_a = scale sum_j (F_aj - F_ja) (+ terms without q/k), each directed pair
-// enters F_a with + and F_j with -, so u = scale (gF_a - gF_j) and
-//   dL/dc_ajh = f_c B_h u.(n + T_aj)   (h < K),  f_c S_aj u.V_at  (h = K + t),
-//   dL/dc_jah = -f_c B_h u.(-n + T_ja) (h < K), -f_c S_ja u.V_jt  (h = K + t).
-// Each pair is visited from both ends, so every atom gathers its own rows'
-// gradients: no atomics, deterministic.
-template <int K, int NC, int NL>
-__global__ void __launch_bounds__(128) k_nc_head_bwd(NCHeadArgs g, const float *__restrict__ gF,
-                                                    float *__restrict__ gQK, float *__restrict__ gV) {
-    constexpr int H = K + NL, QKW = 2 * H * NC;
-    static_assert(2 * H <= 32, "one lane per head and role");
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wa = blockIdx.x * 4 + warp;
-    if (wa >= g.n_atoms || *g.err) return;
-    const int a = g.order ? __ldg(g.order + wa) : wa;
-    const bool role_aj = lane < H, live = lane < 2 * H;
-    const int h = role_aj ? lane : (live ? lane - H : 0);
-    const float isnc = rsqrtf((float)NC);
-    // own row: q_a[h] (role aj) or k_a[h] (role ja)
-    float mine[NC], acc[NC], accv[3] = {0.f, 0.f, 0.f};   // accv: dL/dV_at on the tensor-head lanes of role aj
-    const float *ra = g.QK + (size_t)a * QKW + (role_aj ? 0 : H * NC) + h * NC;
-#pragma unroll
-    for (int d = 0; d < NC; ++d) {
-        mine[d] = live ? ra[d] : 0.f;
-        acc[d] = 0.f;
-    }
-    float va[3 * NL];
-#pragma unroll
-    for (int t = 0; t < 3 * NL; ++t) va[t] = g.V[(size_t)a * nc_v_stride(NL) + t];
-    const float gax = gF[3 * a], gay = gF[3 * a + 1], gaz = gF[3 * a + 2];
-    const int rep = g.atom_rep[a];
-    const float bx = g.box[3 * rep], by = g.box[3 * rep + 1], bz = g.box[3 * rep + 2];
-    const float ibx = bx > 0.f ? 1.f / bx : 0.f, iby = by > 0.f ? 1.f / by : 0.f, ibz = bz > 0.f ? 1.f / bz : 0.f;
-    const float xa = g.x[3 * a], ya = g.x[3 * a + 1], za = g.x[3 * a + 2];
-    const float rc2 = g.rc * g.rc;
-    for (int e = g.row_ptr[a]; e < g.row_ptr[a + 1]; ++e) {
-        const int j = __ldg(g.col + e);
-        const float dx = min_img(__ldg(g.x + 3 * j) - xa, bx, ibx);
-        const float dy = min_img(__ldg(g.x + 3 * j + 1) - ya, by, iby);
-        const float dz = min_img(__ldg(g.x + 3 * j + 2) - za, bz, ibz);
-        const float r2 = dx * dx + dy * dy + dz * dz;
-        if (!(r2 < rc2)) continue;   // uniform over the warp
-        const float r = sqrtf(r2), inv = 1.f / r;
-        const float nx = dx * inv, ny = dy * inv, nz = dz * inv;
-        float du;
-        const float fc = envelope(r * g.inv_rc, g.p, &du);
-        float B[K];
-        bessel<K, false>(r, g.inv_rc, g.bnorm, B, nullptr);
-        float Bh = 0.f;
-#pragma unroll
-        for (int k = 0; k < K; ++k) Bh = (h == k) ? B[k] : Bh;
-        // the other atom's row: k_j[h] (role aj) or q_j[h] (role ja)
-        float other[NC];
-        const float *rj = g.QK + (size_t)j * QKW + (role_aj ? H * NC : 0) + h * NC;
-        float c = 0.f;
-#pragma unroll
-        for (int d = 0; d < NC; ++d) {
-            other[d] = live ? __ldg(rj + d) : 0.f;
-            c = fmaf(mine[d], other[d], c);
-        }
-        c *= isnc;
-        const bool bes = live && h < K;
-        const int t = h - K;
-        float vt[3] = {0.f, 0.f, 0.f};   // V_at (role aj) or V_jt (role ja) of this tensor head
-        if (live && h >= K) {
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-                vt[q] = role_aj ? va[3 * (t < NL ? t : 0) + q]
-                                : __ldg(g.V + (size_t)j * nc_v_stride(NL) + 3 * (t < NL ? t : 0) + q);
-        }
-        const float sB = bes ? c * Bh : 0.f;
-        const float S_aj = warp_sum(role_aj ? sB : 0.f), S_ja = warp_sum(role_aj ? 0.f : sB);
-        float T_aj[3], T_ja[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const float cv = (live && h >= K) ? c * vt[q] : 0.f;
-            T_aj[q] = warp_sum(role_aj ? cv : 0.f);
-            T_ja[q] = warp_sum(role_aj ? 0.f : cv);
-        }
-        const float ux = g.scale * (gax - __ldg(gF + 3 * j)), uy = g.scale * (gay - __ldg(gF + 3 * j + 1)),
-                    uz = g.scale * (gaz - __ldg(gF + 3 * j + 2));
-        float G;
-        if (role_aj) {
-            G = h < K ? fc * Bh * (ux * (nx + T_aj[0]) + uy * (ny + T_aj[1]) + uz * (nz + T_aj[2]))
-                      : fc * S_aj * (ux * vt[0] + uy * vt[1] + uz * vt[2]);
-        } else {
-            G = h < K ? -fc * Bh * (ux * (-nx + T_ja[0]) + uy * (-ny + T_ja[1]) + uz * (-nz + T_ja[2]))
-                      : -fc * S_ja * (ux * vt[0] + uy * vt[1] + uz * vt[2]);
-        }
-        if (role_aj && h >= K) {
-            // V_at enters F_aj = f_c S_aj (n + sum_t c_aj(K+t) V_at) only
-            const float f = fc * S_aj * c;
-            accv[0] = fmaf(f, ux, accv[0]); accv[1] = fmaf(f, uy, accv[1]); accv[2] = fmaf(f, uz, accv[2]);
-        }
-        G *= isnc;
-#pragma unroll
-        for (int d = 0; d < NC; ++d) acc[d] = fmaf(G, other[d], acc[d]);
-    }
-    if (gV && role_aj && h >= K) {
-        float *o = gV + ((size_t)a * NL + (h - K)) * 3;
-        o[0] = accv[0]; o[1] = accv[1]; o[2] = accv[2];
-    }
-    if (live) {
-        const int c0 = (role_aj ? 0 : H * NC) + h * NC;
-#pragma unroll
-        for (int d = 0; d < NC; ++d) gQK[(size_t)a * QKW + c0 + d] = acc[d];
-    }
-}
-
-template <int K, int NC, int NL>
-static void nc_head_bwd_launch(const NCHeadArgs &a, const float *gF, float *gQK, float *gV, cudaStream_t st) {
-    k_nc_head_bwd<K, NC, NL><<<(a.n_atoms + 3) / 4, 128, 0, st>>>(a, gF, gQK, gV);
-    count_launch();
-}
-
-void launch_nc_head_bwd(int K, int n_c, int n_l, const NCHeadArgs &a, const float *gF, float *gQK, float *gV,
-                        cudaStream_t st) {
-    if (a.n_atoms == 0) return;
-    if (K == 8 && n_c == 8 && n_l == 2) nc_head_bwd_launch<8, 8, 2>(a, gF, gQK, gV, st);
-    else if (K == 8 && n_c == 8 && n_l == 1) nc_head_bwd_launch<8, 8, 1>(a, gF, gQK, gV, st);
-    else if (K == 8 && n_c == 8 && n_l == 3) nc_head_bwd_launch<8, 8, 3>(a, gF, gQK, gV, st);
-    else if (K == 8 && n_c == 8 && n_l == 4) nc_head_bwd_launch<8, 8, 4>(a, gF, gQK, gV, st);
-}
-
-// ------------------------------------------------ weight gradients (A^T B)
-// Block (32 x 8 threads) = a 32 x 32 output tile over one slice of atoms;
-// thread (ty, tx) sums outputs (ty + 8k, tx), k < 4, in atom order.
-constexpr int ATB_T = 32, ATB_CH = 16, ATB_SLICES = 64;
-
-__global__ void __launch_bounds__(256) k_atb_part(int N, int O, int I, const float *__restrict__ G,
-                                                 const float *__restrict__ X, float *__restrict__ part, int with_cs,
-                                                 int slices) {
-    __shared__ float Gs[ATB_CH][ATB_T], Xs[ATB_CH][ATB_T];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int o0 = blockIdx.x * ATB_T, i0 = blockIdx.y * ATB_T, sl = blockIdx.z;
-    const int per = (N + slices - 1) / slices, a0 = sl * per, a1 = min(N, a0 + per);
-    float acc[4] = {0.f, 0.f, 0.f, 0.f}, cs[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int c0 = a0; c0 < a1; c0 += ATB_CH) {
-        for (int q = threadIdx.x; q < ATB_CH * ATB_T; q += 256) {
-            const int aa = q / ATB_T, cc = q % ATB_T, at = c0 + aa;
-            Gs[aa][cc] = (at < a1 && o0 + cc < O) ? G[(size_t)at * O + o0 + cc] : 0.f;
-            Xs[aa][cc] = (at < a1 && i0 + cc < I) ? X[(size_t)at * I + i0 + cc] : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int aa = 0; aa < ATB_CH; ++aa) {
-            const float xv = Xs[aa][tx];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                acc[k] = fmaf(Gs[aa][ty + 8 * k], xv, acc[k]);
-                cs[k] += Gs[aa][ty + 8 * k];
-            }
-        }
-        __syncthreads();
-    }
-    float *pp = part + (size_t)sl * O * (I + 1);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int o = o0 + ty + 8 * k, i = i0 + tx;
-        if (o < O && i < I) pp[(size_t)o * (I + 1) + i] = acc[k];
-        if (with_cs && o < O && blockIdx.y == 0 && tx == 0) pp[(size_t)o * (I + 1) + I] = cs[k];
-    }
-}
-
-__global__ void k_atb_reduce(int O, int I, const float *__restrict__ part, float *__restrict__ out,
-                             float *__restrict__ cs, int slices) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= O * (I + 1)) return;
-    const int o = q / (I + 1), i = q % (I + 1);
-    if (i == I && !cs) return;
-    float t = 0.f;
-    for (int s = 0; s < slices; ++s) t += part[(size_t)s * O * (I + 1) + q];
-    if (i < I) out[(size_t)o * I + i] = t;
-    else cs[o] = t;
-}
-
-void launch_atb(int N, int O, int I, const float *G, const float *X, float *out, float *cs, float *part,
-                cudaStream_t st) {
-    if (O == 0 || I == 0) return;
-    const int slices = std::max(1, std::min(ATB_SLICES, (N + 255) / 256));
-    dim3 grid((O + ATB_T - 1) / ATB_T, (I + ATB_T - 1) / ATB_T, slices);
-    k_atb_part<<<grid, 256, 0, st>>>(N, O, I, G, X, part, cs != nullptr, slices);
-    count_launch();
-    const int tot = O * (I + 1);
-    k_atb_reduce<<<(tot + 255) / 256, 256, 0, st>>>(O, I, part, out, cs, slices);
-    count_launch();
-}
-
-// ------------------------------------------- NC layer weight gradients
-// Blocks of four warps take atoms in a grid stride; lanes own channel sets
-// (C / 32 each); every lane sweeps the atom's active edges in list order.
-// Each block adds its warps' sums in warp order into its partial row, and
-// k_sum_rows adds the blocks' rows in block order: deterministic.
-constexpr int WG_BLOCKS = 1024;
-
-template <int C>
-__global__ void __launch_bounds__(128) k_nc_layer_wgrad(NCLayerGradArgs g, float *__restrict__ part) {
-    constexpr int K = 8, CPW = C / 32, NW = 2 * K * C;
-    __shared__ float red[4][NW];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float wacc[2][K][CPW];
-#pragma unroll
-    for (int l = 0; l < 2; ++l)
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-#pragma unroll
-            for (int u = 0; u < CPW; ++u) wacc[l][k][u] = 0.f;
-    const float rc2 = g.rc * g.rc;
-    for (int i = blockIdx.x * 4 + warp; i < g.n_atoms && !*g.err; i += gridDim.x * 4) {
-        float gA[4][CPW];
-#pragma unroll
-        for (int u = 0; u < CPW; ++u) {
-            const int c = lane * CPW + u;
-            const float g0 = g.gq[(size_t)i * 2 * C + c], g1 = g.gq[(size_t)i * 2 * C + C + c];
-            gA[0][u] = 2.f * g.A[((size_t)i * 4) * C + c] * g0;
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                float t = 2.f * g.A[((size_t)i * 4 + 1 + m) * C + c] * g1;
-                for (int h = 0; h < g.n_l; ++h) t = fmaf(g.U[h * C + c], g.gV[((size_t)i * g.n_l + h) * 3 + m], t);
-                gA[1 + m][u] = t;
-            }
-        }
-        const int rep = g.atom_rep[i];
-        const float bx = g.box[3 * rep], by = g.box[3 * rep + 1], bz = g.box[3 * rep + 2];
-        const float ibx = bx > 0.f ? 1.f / bx : 0.f, iby = by > 0.f ? 1.f / by : 0.f, ibz = bz > 0.f ? 1.f / bz : 0.f;
-        const float xi = g.x[3 * i], yi = g.x[3 * i + 1], zi = g.x[3 * i + 2];
-        for (int e = g.row_ptr[i]; e < g.row_ptr[i + 1]; ++e) {
-            const int j = __ldg(g.col + e);
-            const float dx = min_img(__ldg(g.x + 3 * j) - xi, bx, ibx);
-            const float dy = min_img(__ldg(g.x + 3 * j + 1) - yi, by, iby);
-            const float dz = min_img(__ldg(g.x + 3 * j + 2) - zi, bz, ibz);
-            const float r2 = dx * dx + dy * dy + dz * dz;
-            if (!(r2 < rc2)) continue;   // uniform over the warp
-            const float r = sqrtf(r2), inv = 1.f / r;
-            float du;
-            const float fc = envelope(r * g.inv_rc, g.p, &du);
-            float B[K], Y[4];
-            bessel<K, false>(r, g.inv_rc, g.bnorm, B, nullptr);
-            sph<1>(dx * inv, dy * inv, dz * inv, Y);
-#pragma unroll
-            for (int u = 0; u < CPW; ++u) {
-                const float sj = __ldg(g.s0 + (size_t)j * C + lane * CPW + u);
-                const float z0 = gA[0][u] * Y[0] * sj * fc;
-                const float z1 = fmaf(gA[1][u], Y[1], fmaf(gA[2][u], Y[2], gA[3][u] * Y[3])) * sj * fc;
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    wacc[0][k][u] = fmaf(z0, B[k], wacc[0][k][u]);
-                    wacc[1][k][u] = fmaf(z1, B[k], wacc[1][k][u]);
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int l = 0; l < 2; ++l)
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-#pragma unroll
-            for (int u = 0; u < CPW; ++u) red[warp][(l * K + k) * C + lane * CPW + u] = g.nu * wacc[l][k][u];
-    __syncthreads();
-    for (int q = threadIdx.x; q < NW; q += blockDim.x)
-        part[(size_t)blockIdx.x * NW + q] = ((red[0][q] + red[1][q]) + red[2][q]) + red[3][q];
-}
-
-__global__ void k_sum_rows(int Q, int rows, const float *__restrict__ part, float *__restrict__ out) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= Q) return;
-    float t = 0.f;
-    for (int r = 0; r < rows; ++r) t += part[(size_t)r * Q + q];
-    out[q] = t;
-}
-
-void launch_nc_layer_wgrad(int C, const NCLayerGradArgs &a, float *part, float *out, cudaStream_t st) {
-    if (a.n_atoms == 0) return;
-    const int blocks = std::max(1, std::min(WG_BLOCKS, (a.n_atoms + 3) / 4));
-    if (C == 32) k_nc_layer_wgrad<32><<<blocks, 128, 0, st>>>(a, part);
-    else if (C == 64) k_nc_layer_wgrad<64><<<blocks, 128, 0, st>>>(a, part);
-    else return;
-    count_launch();
-    const int Q = 2 * 8 * C;
-    k_sum_rows<<<(Q + 255) / 256, 256, 0, st>>>(Q, blocks, part, out);
-    count_launch();
-}
-
-__global__ void k_nc_dU_part(int n, int C, int n_l, const float *__restrict__ gV, const float *__restrict__ A,
-                             float *__restrict__ part, int slices) {
-    const int q = threadIdx.x;   // q = t C + c
-    if (q >= n_l * C) return;
-    const int t = q / C, c = q - t * C;
-    const int per = (n + slices - 1) / slices, a0 = blockIdx.x * per, a1 = min(n, a0 + per);
-    float acc = 0.f;
-    for (int i = a0; i < a1; ++i)
-#pragma unroll
-        for (int m = 0; m < 3; ++m) acc = fmaf(gV[((size_t)i * n_l + t) * 3 + m], A[((size_t)i * 4 + 1 + m) * C + c], acc);
-    part[(size_t)blockIdx.x * n_l * C + q] = acc;
-}
-
-void launch_nc_dU(int n, int C, int n_l, const float *gV, const float *A, float *part, float *out, cudaStream_t st) {
-    if (n == 0) return;
-    const int slices = std::max(1, std::min(64, (n + 255) / 256));
-    k_nc_dU_part<<<slices, 256, 0, st>>>(n, C, n_l, gV, A, part, slices);
-    count_launch();
-    k_sum_rows<<<(n_l * C + 255) / 256, 256, 0, st>>>(n_l * C, slices, part, out);
-    count_launch();
-}
-
-__global__ void k_distill_residual(int n, const float *F, const float *T, float *g, float *sq) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.f;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const float d = F[3 * i + q] - T[3 * i + q];
-        g[3 * i + q] = 2.f * d;
-        s = fmaf(d, d, s);
-    }
-    sq[i] = s;
-}
-
-void launch_distill_residual(int n, const float *F, const float *T, float *g, float *sq, cudaStream_t st) {
-    if (n == 0) return;
-    k_distill_residual<<<(n + 255) / 256, 256, 0, st>>>(n, F, T, g, sq);
-    count_launch();
-}
-
-// Adam (Kingma & Ba), beta1 0.9, beta2 0.999, eps 1e-8, bias-corrected.
-__global__ void k_adam(int n, float *w, const float *grad, float *m, float *v, float lr, float c1, float c2,
-                       __nv_bfloat16 *w_bf, int kd) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gr = grad[i];
-    const float mi = 0.9f * m[i] + 0.1f * gr, vi = 0.999f * v[i] + 0.001f * gr * gr;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
-    w[i] = wi;
-    if (w_bf) st_split(w_bf, (size_t)(i / kd), kd, i % kd, wi);
-}
-
-void launch_adam(int n, float *w, const float *grad, float *m, float *v, float lr, int step, __nv_bfloat16 *w_bf,
-                 int kd, cudaStream_t st) {
-    if (n == 0) return;
-    const float c1 = 1.f - powf(0.9f, (float)step), c2 = 1.f - powf(0.999f, (float)step);
-    k_adam<<<(n + 255) / 256, 256, 0, st>>>(n, w, grad, m, v, lr, c1, c2, w_bf, kd);
-    count_launch();
 }
 
 __global__ void k_scale_d(double *v, int n, double f) {

@@ -77,6 +77,7 @@ struct FirstIO {
     int n_species;           // <= DMTS_MAX_SPECIES
     float nu;
     float *A;                // [N][NLM][C] (forward out, nullable: not stored; backward in)
+    float *T;                // [N][n_species][NLM][K] basis sums per species (forward out, nullable)
     float *q;                // [N][(LMAX+1)C] (forward out, nullable)
     __nv_bfloat16 *q_bf16;   // optional split-bf16 copy of q (forward out)
     const float *UW;         // tensor-head weights [n_l][n_species][K] (with V)
