@@ -970,6 +970,17 @@ dmts_status nbr_build(dmts_ctx *ctx, const dmts_system *sys, dmts_nbr *nbr, long
         if (n_pairs) *n_pairs = 0;
         return DMTS_OK;
     }
+    // Rows kept sorted by the count, so that the fill copies them instead of
+    // sweeping and sorting again (12,288 atoms: count and fill 28 + 75 us -> 36 + 9).
+    // Larger systems, and one whose scratch cannot be had, sweep again.
+    if ((long long)sys->n_atoms <= kNbrSlotAtoms) {
+        if (ctx->nbr_scratch.slots.ensure(sizeof(int) * (size_t)sys->n_atoms * kNbrSlots)) {
+            nw.slots = (int *)ctx->nbr_scratch.slots.p;
+            nw.slot_cap = kNbrSlots;
+        } else {
+            cudaGetLastError();   // the build goes on without it
+        }
+    }
     nbr_cells(nw, nbr->r_list, st);
     nbr_fill(nw, nbr->r_list, nbr->row_ptr, nbr->col, nbr->capacity, nullptr, st);
     long long tot = 0;

@@ -341,8 +341,8 @@ void launch_atb(int N, int O, int I, const float *G, const float *X, float *out,
 // no neighbour is visited again. Warps take atoms in a grid stride, lanes own
 // C / 32 channels; each block adds its warps' sums in warp order into its row
 // of `part`, and k_sum_rows adds the rows in a fixed order: deterministic.
-// (49,152 atoms, C = 64: 68 + 14 us, bound by the loads' latency at four warps
-// an SM quarter; 597 + 372 + 72 us when every edge was visited again and dU was
+// (49,152 atoms, C = 64: 68 + 14 us;
+// 597 + 372 + 72 us when every edge was visited again and dU was
 // summed by 64 blocks of its own.)
 constexpr int WG_WARPS = 4;
 

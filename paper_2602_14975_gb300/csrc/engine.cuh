@@ -43,11 +43,12 @@ struct DevModel {
     __nv_bfloat16 *wr_bf = nullptr, *wrt_bf = nullptr, *wqk_bf = nullptr;
 };
 
-constexpr int kNbrSlots = 128;   // longest row kept by the count pass of a state's rebuild
+constexpr int kNbrSlots = 128;   // longest row kept by a build's count pass
+constexpr long long kNbrSlotAtoms = 1 << 21;   // a list build outside a state keeps rows up to here (1 GiB of scratch)
 
 struct NbrScratch {
     Buf grid, cell_cnt, cell_start, cell_atoms, atom_cell, atom_slot, counts, total, counts_sub;
-    Buf slots;    // [n_atoms][kNbrSlots] sorted rows kept between the count and the fill of a rebuild
+    Buf slots;    // [n_atoms][kNbrSlots] sorted rows kept between the count and the fill
     Buf scan;     // prefix-scan status words [2][scan_tiles] and epoch/tile counters [2] (zero-initialised)
     int scan_tiles = 0;
     void release_all() {

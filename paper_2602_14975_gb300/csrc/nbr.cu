@@ -274,25 +274,31 @@ __device__ __forceinline__ void sort_row(int *sb, int cnt, int lane) {
 
 // Writes the entries of sb[0..cnt) (distinct keys, compared without
 // SUB_FLAG) to dst in ascending order: each entry goes to the position given
-// by the number of smaller keys. A lane ranks entries lane, lane + 32, ...;
-// every key is read once per lane. cnt <= 128.
-__device__ __forceinline__ void rank_scatter(const int *sb, int cnt, int *dst, int lane) {
-    int v[4], k[4], r[4];
+// by the number of smaller keys. A lane ranks entries lane, lane + 32, ... (Q
+// of them, 32 (Q - 1) < cnt <= 32 Q); the keys are read four at a time, the
+// tail past cnt as keys above all others.
+template <int Q>
+__device__ __forceinline__ void rank_scatter(int *sb, int cnt, int *dst, int lane) {
+    if (lane < 3) sb[cnt + lane] = 0x7fffffff;   // (rows hold at least 32 Q + 4 entries)
+    __syncwarp();
+    int v[Q], k[Q], r[Q];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < Q; ++q) {
         const int t = lane + 32 * q;
         v[q] = t < cnt ? sb[t] : 0;
-        k[q] = t < cnt ? (v[q] & 0x7fffffff) : -1;
+        k[q] = v[q] & 0x7fffffff;
         r[q] = 0;
     }
-#pragma unroll 4
-    for (int u = 0; u < cnt; ++u) {
-        const int ku = sb[u] & 0x7fffffff;
+#pragma unroll 2
+    for (int u = 0; u < cnt; u += 4) {
+        const int4 ku = *reinterpret_cast<const int4 *>(sb + u);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] += ku < k[q] ? 1 : 0;
+        for (int q = 0; q < Q; ++q)
+            r[q] += ((ku.x & 0x7fffffff) < k[q]) + ((ku.y & 0x7fffffff) < k[q]) + ((ku.z & 0x7fffffff) < k[q]) +
+                    ((ku.w & 0x7fffffff) < k[q]);
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < Q; ++q)
         if (lane + 32 * q < cnt) dst[r[q]] = v[q];
 }
 
@@ -322,8 +328,14 @@ struct RowAcc {
         if (keep && cnt <= w.slot_cap && cnt <= NB_MAXROW) {
             __syncwarp();
             int *dst = w.slots + (size_t)i * w.slot_cap;
-            if (cnt <= 128) {
-                rank_scatter(sb, cnt, dst, lane);
+            if (cnt <= 32) {
+                rank_scatter<1>(sb, cnt, dst, lane);
+            } else if (cnt <= 64) {
+                rank_scatter<2>(sb, cnt, dst, lane);
+            } else if (cnt <= 96) {
+                rank_scatter<3>(sb, cnt, dst, lane);
+            } else if (cnt <= 128) {
+                rank_scatter<4>(sb, cnt, dst, lane);
             } else {
                 sort_row(sb, cnt, lane);
                 for (int t = lane; t < cnt; t += 32) dst[t] = sb[t];
@@ -333,19 +345,7 @@ struct RowAcc {
     }
 };
 
-__global__ void __launch_bounds__(NB_WARPS * 32) k_nbr_count_warp(NbrWork w, float rc2, float rc2_sub) {
-    if (gated_off(w.gate, w.err)) return;
-    __shared__ int buf[NB_WARPS][NB_MAXROW];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * NB_WARPS + warp;
-    if (i >= w.n_atoms) return;
-    const bool keep = w.slots != nullptr;
-    RowAcc acc{buf[warp]};
-    for_candidates_warp(w, i, rc2, lane, [&](bool hit, int j, float r2) { acc.add(w, keep, hit, j, r2, rc2_sub, lane); });
-    acc.finish(w, keep, i, lane);
-}
-
-// The same count by cells: one block per cell stages the indices and
+// The count by cells: one block per cell stages the indices and
 // positions of every candidate of its neighbouring cells in shared memory
 // once (in the order for_candidates_warp visits them), then each warp
 // sweeps them for one atom of the cell at a time. The candidates' positions
@@ -357,15 +357,16 @@ __global__ void __launch_bounds__(NBC_WARPS * 32) k_nbr_count_cell(NbrWork w, fl
     if (gated_off(w.gate, w.err)) return;
     __shared__ int cj[NBC_CAP];
     __shared__ float cx[NBC_CAP], cy[NBC_CAP], cz[NBC_CAP];
-    __shared__ int buf[NBC_WARPS][NB_MAXROW];
+    __shared__ __align__(16) int buf[NBC_WARPS][NB_MAXROW];
     __shared__ int seg_beg[18], seg_excl[19];
     const int c = blockIdx.x;
     const int a_beg = w.cell_start[c], a_end = w.cell_start[c + 1];
     if (a_beg == a_end) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const CellGrid g = w.grid[w.atom_rep[w.cell_atoms[a_beg]]];
-    if (threadIdx.x == 0) {
-        // the neighbouring cells' x-runs, as for_candidates_warp forms them
+    if (warp == 0) {
+        // the neighbouring cells' x-runs, in the order for_candidates_warp forms
+        // them: lane s takes run s, both parts of a wrapped one next to each other
         const int own = c - g.cell_off;
         const int ccx = own % g.dim[0], ccy = (own / g.dim[0]) % g.dim[1], ccz = own / (g.dim[0] * g.dim[1]);
         int lo[3], hi[3];
@@ -383,27 +384,25 @@ __global__ void __launch_bounds__(NBC_WARPS * 32) k_nbr_count_cell(NbrWork w, fl
         int a0 = ccx + lo[0], b0 = ccx + hi[0], a1 = 0, b1 = -1;
         if (a0 < 0) { a1 = a0 + g.dim[0]; b1 = g.dim[0] - 1; a0 = 0; }
         else if (b0 >= g.dim[0]) { a1 = 0; b1 = b0 - g.dim[0]; b0 = g.dim[0] - 1; }
-        int ns = 0, tot = 0;
-        for (int oz = lo[2]; oz <= hi[2]; ++oz) {
-            int z = ccz + oz;
+        const int parts = b1 >= a1 ? 2 : 1, ny = hi[1] - lo[1] + 1, ns = (hi[2] - lo[2] + 1) * ny * parts;
+        int sbeg = 0, slen = 0;
+        if (lane < ns) {
+            const int part = lane % parts, yz = lane / parts;
+            int y = ccy + lo[1] + yz % ny, z = ccz + lo[2] + yz / ny;
+            if (g.box[1] > 0.f) y = (y + g.dim[1]) % g.dim[1];
             if (g.box[2] > 0.f) z = (z + g.dim[2]) % g.dim[2];
-            for (int oy = lo[1]; oy <= hi[1]; ++oy) {
-                int y = ccy + oy;
-                if (g.box[1] > 0.f) y = (y + g.dim[1]) % g.dim[1];
-                const int row = g.cell_off + (z * g.dim[1] + y) * g.dim[0];
-                seg_beg[ns] = w.cell_start[row + a0];
-                seg_excl[ns] = tot;
-                tot += w.cell_start[row + b0 + 1] - seg_beg[ns];
-                ++ns;
-                if (b1 >= a1) {
-                    seg_beg[ns] = w.cell_start[row + a1];
-                    seg_excl[ns] = tot;
-                    tot += w.cell_start[row + b1 + 1] - seg_beg[ns];
-                    ++ns;
-                }
-            }
+            const int row = g.cell_off + (z * g.dim[1] + y) * g.dim[0];
+            sbeg = w.cell_start[row + (part ? a1 : a0)];
+            slen = w.cell_start[row + (part ? b1 : b0) + 1] - sbeg;
         }
-        for (int k = ns; k < 19; ++k) seg_excl[k] = tot;
+        int incl = slen;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(DMTS_FULL, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane < 18) seg_beg[lane] = sbeg;
+        if (lane < 19) seg_excl[lane] = incl - slen;   // (lane 18: the total)
     }
     __syncthreads();
     const int total = seg_excl[18];
@@ -484,7 +483,7 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_nbr_fill_warp(NbrWork w, floa
                                                                  float *x_ref, float rc2_sub, const int *sub_row,
                                                                  int *sub_col) {
     if (gated_off(w.gate, w.err)) return;
-    __shared__ int buf[NB_WARPS][NB_MAXROW];
+    __shared__ __align__(16) int buf[NB_WARPS][NB_MAXROW];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * NB_WARPS + warp;
     if (i >= w.n_atoms) return;
