@@ -53,6 +53,23 @@ bool Buf::ensure(size_t bytes) {
     return true;
 }
 
+void *PinnedBuf::ensure(size_t bytes) {
+    if (bytes <= cap) return p;
+    release();
+    if (cudaMallocHost(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+        return nullptr;
+    }
+    cap = bytes;
+    return p;
+}
+void PinnedBuf::release() {
+    if (p) cudaFreeHost(p);
+    p = nullptr;
+    cap = 0;
+}
+
 // ensure() for a buffer that must hold zeros whenever it is not in use: a
 // new allocation is cleared on the stream.
 static bool ensure_zeroed(dmts_ctx *ctx, Buf &b, size_t bytes, cudaStream_t st) {
@@ -685,13 +702,21 @@ void prepare_nbr_work_async(dmts_ctx *ctx, StateInternal *si, const SysView &v, 
 // Stream-ordered host copies of the replica offsets and boxes.
 static bool host_copy_offsets(dmts_ctx *ctx, const dmts_system *sys, std::vector<int> &rep_off,
                               std::vector<float> &box, cudaStream_t st) {
-    rep_off.resize(sys->n_replicas + 1);
-    box.resize(3 * sys->n_replicas);
-    return ck(ctx, cudaMemcpyAsync(rep_off.data(), sys->rep_off, sizeof(int) * rep_off.size(), cudaMemcpyDeviceToHost, st),
-              "rep_off copy") &&
-           ck(ctx, cudaMemcpyAsync(box.data(), sys->box, sizeof(float) * box.size(), cudaMemcpyDeviceToHost, st),
-              "box copy") &&
-           ck(ctx, cudaStreamSynchronize(st), "offsets");
+    const size_t nr = (size_t)sys->n_replicas;
+    rep_off.resize(nr + 1);
+    box.resize(3 * nr);
+    // through pinned memory: both copies in flight, one wait (a copy to pageable
+    // memory waits by itself: a list build of 12,288 atoms: 155 -> 130 us with the same for its results)
+    unsigned char *h = (unsigned char *)ctx->pinned.ensure(std::max<size_t>(kPinnedBytes, sizeof(int) * (nr + 1) + sizeof(float) * 3 * nr));
+    if (!h) { fail(ctx, DMTS_E_OOM, "pinned staging allocation failed"); return false; }
+    const size_t nb = sizeof(int) * (nr + 1);
+    if (!ck(ctx, cudaMemcpyAsync(h, sys->rep_off, nb, cudaMemcpyDeviceToHost, st), "rep_off copy") ||
+        !ck(ctx, cudaMemcpyAsync(h + nb, sys->box, sizeof(float) * 3 * nr, cudaMemcpyDeviceToHost, st), "box copy") ||
+        !ck(ctx, cudaStreamSynchronize(st), "offsets"))
+        return false;
+    memcpy(rep_off.data(), h, nb);
+    memcpy(box.data(), h + nb, sizeof(float) * 3 * nr);
+    return true;
 }
 
 // Prefix-scan scratch for scans of up to n elements (status words and tile
@@ -720,8 +745,9 @@ static dmts_status prepare_nbr_work(dmts_ctx *ctx, NbrScratch &b, const SysView 
         !b.counts.ensure(sizeof(int) * (N + 1)) || !b.counts_sub.ensure(sizeof(int) * (N + 1)) ||
         !b.total.ensure(sizeof(long long)))
         return fail(ctx, DMTS_E_OOM, "neighbour scratch allocation failed");
-    if (!ck(ctx, cudaMemcpyAsync(b.grid.p, grids.data(), sizeof(CellGrid) * R, cudaMemcpyHostToDevice, st), "grid upload") ||
-        !ck(ctx, cudaStreamSynchronize(st), "grid upload"))
+    if (!scan_scratch(ctx, b, std::max(N, n_cells), nw, st)) return fail(ctx, DMTS_E_OOM, "scan scratch allocation failed");
+    // (`grids` outlives the caller's next wait on the stream)
+    if (!ck(ctx, cudaMemcpyAsync(b.grid.p, grids.data(), sizeof(CellGrid) * R, cudaMemcpyHostToDevice, st), "grid upload"))
         return DMTS_E_CUDA;
     nw.n_atoms = N;
     nw.n_rep = R;
@@ -740,7 +766,6 @@ static dmts_status prepare_nbr_work(dmts_ctx *ctx, NbrScratch &b, const SysView 
     nw.total = (long long *)b.total.p;
     nw.gate = gate;
     nw.err = ctx->d_err;
-    if (!scan_scratch(ctx, b, std::max(N, n_cells), nw, st)) return fail(ctx, DMTS_E_OOM, "scan scratch allocation failed");
     return DMTS_OK;
 }
 
@@ -845,6 +870,7 @@ dmts_status dmts_create(dmts_ctx **out, const dmts_model *cons, const dmts_model
         return fail(nullptr, DMTS_E_OOM, "allocation failed");
     }
     cudaMemset(ctx->d_err, 0, sizeof(int));
+    ctx->pinned.ensure(kPinnedBytes);   // (tried again at its first use)
     if (cons) {
         dmts_status s = load_model(ctx, cons, false, ctx->cons);
         if (s != DMTS_OK) {
@@ -892,6 +918,7 @@ void dmts_destroy(dmts_ctx *ctx) {
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
     ctx->ws.release_all();
     ctx->nbr_scratch.release_all();
+    ctx->pinned.release();
     ctx->prof.release();
     delete ctx;
 }
@@ -983,13 +1010,13 @@ dmts_status nbr_build(dmts_ctx *ctx, const dmts_system *sys, dmts_nbr *nbr, long
     }
     nbr_cells(nw, nbr->r_list, st);
     nbr_fill(nw, nbr->r_list, nbr->row_ptr, nbr->col, nbr->capacity, nullptr, st);
-    long long tot = 0;
-    if (!ck(ctx, cudaMemcpyAsync(&tot, nw.total, sizeof(long long), cudaMemcpyDeviceToHost, st), "count copy") ||
+    long long *h = (long long *)ctx->pinned.p;   // pair count, error word (host_copy_offsets has sized it)
+    if (!ck(ctx, cudaMemcpyAsync(h, nw.total, sizeof(long long), cudaMemcpyDeviceToHost, st), "count copy") ||
+        !ck(ctx, cudaMemcpyAsync(h + 1, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, st), "error word") ||
         !ck(ctx, cudaStreamSynchronize(st), "nbr_build"))
         return DMTS_E_CUDA;
-    if (n_pairs) *n_pairs = tot;
-    int err = 0;
-    cudaMemcpy(&err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost);
+    if (n_pairs) *n_pairs = h[0];
+    const int err = *(const int *)(h + 1);
     if (err) {
         cudaMemset(ctx->d_err, 0, sizeof(int));
         if (err == DMTS_E_NBR_OVERFLOW)

@@ -16,6 +16,15 @@ struct Buf {
     bool ensure(size_t bytes);
     void release();
 };
+// Pinned host staging for a call's small copies; a call's last use of it ends
+// with a wait on the call's stream.
+constexpr size_t kPinnedBytes = 64 << 10;   // allocated with the context
+struct PinnedBuf {
+    void *p = nullptr;
+    size_t cap = 0;
+    void *ensure(size_t bytes);   // nullptr on failure
+    void release();
+};
 // Counts the library's device (re)allocations and frees: a captured graph
 // recorded with an older value may hold pointers that are no longer valid.
 unsigned long long alloc_generation();
@@ -165,6 +174,7 @@ struct dmts_ctx {
     std::string last_error;
     dmts::Workspace ws;
     dmts::NbrScratch nbr_scratch;
+    dmts::PinnedBuf pinned;
     dmts::Profiler prof;
     // second stream of respa_step: the NC evaluation at the end of an outer
     // step runs on it, concurrently with the conservative evaluation at the
