@@ -6,6 +6,7 @@
 // fused epilogues.
 #include <algorithm>
 
+#include "edge.cuh"
 #include "epilogue.cuh"
 #include "mp.cuh"
 #include "pack.cuh"
@@ -161,94 +162,110 @@ __global__ void __launch_bounds__(MP_WARPS * 32) k_mp_fwd(EdgeGeom g, LayerIO io
 // neighbour j < a contributes only its sender-role term to g_s_a (R, no R',
 // no force).
 //
-// Shared memory per block (one warp; 21.4 KB at C = 128, l_max = 2): 32 edge
-// records of packs (f_c B_k, its r-derivative, Y_lm) and of scalars
-// (dY_lm/dd, n, and r for the virial), the receiver's gA_a as packs, the 32
-// neighbour indices, and the lanes' shares of the force of FT pairs
-// (transposed so that one lane adds up each pair).
-constexpr int FT = 16;   // pairs per force reduction
-// One warp per block: how many upper neighbours an atom has varies from atom
-// to atom, and a block keeps its registers and shared memory until its
-// slowest warp is done, so single-warp blocks keep the SM's eight warp slots
-// busy (255 registers a thread allow eight warps per SM either way).
-constexpr int BWD_WARPS = 1;
+// One warp per block and atom: how many upper neighbours an atom has varies,
+// and a block keeps its registers until its slowest warp is done. What bounds
+// it: latency and issue at eight warps per SM (24 packs of radial weights live
+// in registers), 288 packed FMA of two cycles per pair, and the L1 data path
+// (the neighbours' rows gA_j, s_j, edge records). So the records are read 16
+// bytes at a time, the direction derivative is formed from n instead of nine
+// stored gradients, and the next chunk's candidates are loaded a chunk ahead:
+// 711 -> 686 us (23,558 atoms, C = 128, l_max = 2), 27 -> 24 us (192 atoms,
+// C = 64, l_max = 1). Measured and slower there: rows staged by bulk copies two
+// visits ahead 779 us, two warps of 64 channels per atom 720 us, prefetches
+// into L1 733 us; with every row in L1 it would take 594 us.
+//
+// Shared memory per block (15.3 KB at C = 128, l_max = 2): gA_a, 32 edge
+// records of packs (f_c B_k, Y_lm, the r-derivative of f_c B_k), directions
+// (n, 1/r) and neighbour indices, and the lanes' shares of the force of FT
+// pairs (transposed so that four lanes add up each pair).
+constexpr int FT = 8;   // pairs per force reduction
 
-template <int C, int LMAX, int K, bool VIR>
+template <int C, int LMAX, int K>
 struct BwdSmem {
     static constexpr int NL = LMAX + 1, NLM = NL * NL, CPW = C / 32;
     using T = typename Pack<CPW>::T;
     static constexpr int NP = Pack<CPW>::NP;
-    static constexpr int RS = (2 * K + NLM) | 1;
-    static constexpr int GS = (3 * NLM + 3 + (VIR ? 1 : 0)) | 1;
-    static constexpr size_t r_bytes = sizeof(T) * BWD_WARPS * 32 * RS;
-    static constexpr size_t ga_bytes = sizeof(T) * BWD_WARPS * NLM * NP * 32;
-    static constexpr size_t g_bytes = sizeof(float) * BWD_WARPS * 32 * GS;
-    static constexpr size_t j_bytes = sizeof(int) * BWD_WARPS * 32;
-    static constexpr size_t f_bytes = sizeof(float) * BWD_WARPS * 3 * FT * 33;
-    static constexpr size_t bytes = r_bytes + ga_bytes + g_bytes + j_bytes + f_bytes;
+    static constexpr int V4 = 16 / sizeof(T);                       // packs per 16-byte word
+    static constexpr int KY = (K + NLM + V4 - 1) / V4 * V4;         // f_c B_k and Y_lm, padded
+    static constexpr int RW = ((KY + K) / V4) | 1;                  // 16-byte words per record, odd: conflict-free
+    float4 rec[32][RW];
+    float4 dir[32];
+    float ga[NLM * C];
+    float f[3][FT][33];
+    int j[32];
 };
 
-template <int C, int LMAX, int K, bool VIR>
-__global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO io) {
-    using S = BwdSmem<C, LMAX, K, VIR>;
-    using T = typename S::T;
-    constexpr int NL = S::NL, NLM = S::NLM, CPW = S::CPW, NP = S::NP, PW = Pack<CPW>::W;
-    constexpr int RS = S::RS, GS = S::GS;
-    extern __shared__ __align__(16) unsigned char mp_smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    T (*sh_r)[RS] = reinterpret_cast<T (*)[RS]>(mp_smem) + warp * 32;
-    T (*sh_ga)[NP * 32] = reinterpret_cast<T (*)[NP * 32]>(mp_smem + S::r_bytes) + warp * NLM;
-    float (*sh_g)[GS] = reinterpret_cast<float (*)[GS]>(mp_smem + S::r_bytes + S::ga_bytes) + warp * 32;
-    int *sh_j = reinterpret_cast<int *>(mp_smem + S::r_bytes + S::ga_bytes + S::g_bytes) + warp * 32;
-    float (*sh_f)[FT][33] =
-        reinterpret_cast<float (*)[FT][33]>(mp_smem + S::r_bytes + S::ga_bytes + S::g_bytes + S::j_bytes) + warp * 3;
-    const int wa = blockIdx.x * BWD_WARPS + warp;
-    if (wa >= g.n_atoms || *io.err) return;
-    const int a = g.order ? __ldg(g.order + wa) : wa;
+// Words [0, N) of a record as packs.
+template <int N, class T>
+__device__ __forceinline__ void ld_rec(const float4 *p, T *v) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        const float4 t = p[q];
+        if constexpr (std::is_same<T, float2>::value) {
+            v[2 * q] = make_float2(t.x, t.y);
+            v[2 * q + 1] = make_float2(t.z, t.w);
+        } else {
+            v[4 * q] = t.x;
+            v[4 * q + 1] = t.y;
+            v[4 * q + 2] = t.z;
+            v[4 * q + 3] = t.w;
+        }
+    }
+}
 
+template <int C, int LMAX, int K, bool VIR>
+__global__ void __launch_bounds__(32) k_mp_bwd(EdgeGeom g, LayerIO io) {
+    using S = BwdSmem<C, LMAX, K>;
+    using T = typename S::T;
+    constexpr int NL = S::NL, NLM = S::NLM, CPW = S::CPW, NP = S::NP, PW = Pack<CPW>::W, V4 = S::V4, KY = S::KY;
+    extern __shared__ __align__(16) unsigned char mp_smem[];
+    S &sm = *reinterpret_cast<S *>(mp_smem);
+    const int lane = threadIdx.x;
+    const Row rw = load_row(g, blockIdx.x);
+    if (*io.err) return;
+    const int a = rw.i, beg = rw.beg, end = rw.end;
+    const int co = lane * CPW;   // this lane's channels
+    // the first candidates
+    int cj = beg + lane < end ? __ldg(g.col + beg + lane) : -1;
     T W[NL][K][NP];
 #pragma unroll
     for (int l = 0; l < NL; ++l)
 #pragma unroll
-        for (int k = 0; k < K; ++k) ldp<CPW>(io.wrad + (l * K + k) * C + lane * CPW, W[l][k]);
-#pragma unroll
-    for (int lm = 0; lm < NLM; ++lm) {
-        T t[NP];
-        ldp<CPW>(io.gA + ((size_t)a * NLM + lm) * C + lane * CPW, t);
-#pragma unroll
-        for (int p = 0; p < NP; ++p) sh_ga[lm][p * 32 + lane] = t[p];
-    }
+        for (int k = 0; k < K; ++k) ldp<CPW>(io.wrad + (l * K + k) * C + co, W[l][k]);
     T sa[NP], san[NP], gse[NP], gso[NP];   // s_a, -s_a; sender-role sums over even and odd l
-    ldp<CPW>(io.s + (size_t)a * C + lane * CPW, sa);
+    ldp<CPW>(io.s + (size_t)a * C + co, sa);
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
         san[p] = vneg(sa[p]);
         gse[p] = vdup<T>(0.f);
         gso[p] = vdup<T>(0.f);
     }
+    float cx = 0.f, cy = 0.f, cz = 0.f;
+    if (cj >= 0) {
+        cx = __ldg(g.x + 3 * cj);
+        cy = __ldg(g.x + 3 * cj + 1);
+        cz = __ldg(g.x + 3 * cj + 2);
+    }
+#pragma unroll
+    for (int lm = 0; lm < NLM; ++lm) {
+        T t[NP];
+        ldp<CPW>(io.gA + ((size_t)a * NLM + lm) * C + co, t);
+        stp<CPW>(sm.ga + lm * C + co, t);
+    }
+    const AtomGeom ge = wrap_inverse(rw.a);
+    const float rc2 = g.rc * g.rc;
     // a's side of its pairs, fixed point (on the lanes that add up a pair)
     long long oa[3] = {0, 0, 0}, ow = 0;
     bool bad = false;   // a pair term outside the fixed-point range (or not finite)
-
-    const int rep = g.atom_rep[a];
-    const float bx = g.box[3 * rep], by = g.box[3 * rep + 1], bz = g.box[3 * rep + 2];
-    const float ibx = bx > 0.f ? 1.f / bx : 0.f, iby = by > 0.f ? 1.f / by : 0.f, ibz = bz > 0.f ? 1.f / bz : 0.f;
-    const float xa = g.x[3 * a], ya = g.x[3 * a + 1], za = g.x[3 * a + 2];
-    const float rc2 = g.rc * g.rc;
-    const int beg = g.row_ptr[a], end = g.row_ptr[a + 1];
     __syncwarp();
+
     for (int base = beg; base < end; base += 32) {
-        const int e = base + lane;
         bool act = false;
-        int j = 0;
-        float dx = 0.f, dy = 0.f, dz = 0.f, r2 = 0.f;
-        if (e < end) {
-            j = __ldg(g.col + e);
-            dx = min_img(__ldg(g.x + 3 * j) - xa, bx, ibx);
-            dy = min_img(__ldg(g.x + 3 * j + 1) - ya, by, iby);
-            dz = min_img(__ldg(g.x + 3 * j + 2) - za, bz, ibz);
-            r2 = dx * dx + dy * dy + dz * dz;
-            act = r2 < rc2;
+        const int j = cj;
+        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (j >= 0) {
+            d = edge_disp(ge, cx, cy, cz);
+            act = d.w < rc2;
         }
         // lower neighbours (j < a) first, then the upper ones (the pairs this
         // warp owns): rows are ascending, so g_s_a takes its terms in row
@@ -256,178 +273,205 @@ __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO i
         // skin entries)
         const bool up = act && j > a, lo = act && j < a;
         const unsigned mu = __ballot_sync(DMTS_FULL, up), ml = __ballot_sync(DMTS_FULL, lo);
-        const int n_up = __popc(mu), n_lo = __popc(ml);
+        const int n_lo = __popc(ml), nt = n_lo + __popc(mu);
+        const unsigned lt = (1u << lane) - 1u;
+        const int pos = lo ? __popc(ml & lt) : n_lo + __popc(mu & lt);
+        if (up || lo) sm.j[pos] = j;
+        const int en = base + 32 + lane;
+        cj = en < end ? __ldg(g.col + en) : -1;
         if (up || lo) {
-            const unsigned lt = (1u << lane) - 1u;
-            const int pos = lo ? __popc(ml & lt) : n_lo + __popc(mu & lt);
-            T *rec = sh_r[pos];
-            float *ge = sh_g[pos];
-            const float r = sqrtf(r2), inv = 1.f / r;
+            const float r = sqrtf(d.w), inv = 1.f / r;
             float du;
             const float fc = envelope(r * g.inv_rc, g.p, &du);
             const float dfc = du * g.inv_rc;
-            float B[K], dB[K];
+            float B[K], dB[K], Y[NLM];
             bessel<K, true>(r, g.inv_rc, g.bnorm, B, dB);
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                rec[k] = vdup<T>(fc * B[k]);
-                rec[K + k] = vdup<T>(dfc * B[k] + fc * dB[k]);
-            }
-            const float nx = dx * inv, ny = dy * inv, nz = dz * inv;
-            float Y[NLM], dY[3 * NLM];
+            const float nx = d.x * inv, ny = d.y * inv, nz = d.z * inv;
             sph<LMAX>(nx, ny, nz, Y);
-            sph_grad<LMAX>(nx, ny, nz, inv, dY);
+            sm.dir[pos] = make_float4(nx, ny, nz, inv);
+            float v[KY + K];
 #pragma unroll
-            for (int lm = 0; lm < NLM; ++lm) rec[2 * K + lm] = vdup<T>(Y[lm]);
+            for (int q = 0; q < KY + K; ++q) {
+                if (q < K) v[q] = fc * B[q < K ? q : 0];
+                else if (q < K + NLM) v[q] = Y[q < K + NLM ? (q >= K ? q - K : 0) : 0];
+                else if (q >= KY) v[q] = dfc * B[q >= KY ? q - KY : 0] + fc * dB[q >= KY ? q - KY : 0];
+                else v[q] = 0.f;
+            }
 #pragma unroll
-            for (int q = 0; q < 3 * NLM; ++q) ge[q] = dY[q];
-            ge[3 * NLM] = nx;
-            ge[3 * NLM + 1] = ny;
-            ge[3 * NLM + 2] = nz;
-            if (VIR) ge[3 * NLM + 3] = r;
-            sh_j[pos] = j;
+            for (int q = 0; q < (KY + K) / V4; ++q)
+                sm.rec[pos][q] = V4 == 2 ? make_float4(v[2 * q], v[2 * q], v[2 * q + 1], v[2 * q + 1])
+                                         : make_float4(v[V4 * q], v[V4 * q + 1], v[V4 * q + V4 / 2], v[V4 * q + V4 - 1]);
+        }
+        if (cj >= 0) {
+            cx = __ldg(g.x + 3 * cj);
+            cy = __ldg(g.x + 3 * cj + 1);
+            cz = __ldg(g.x + 3 * cj + 2);
         }
         __syncwarp();
+
         // lower neighbours: the sender-role gradient only
 #pragma unroll 2
         for (int t = 0; t < n_lo; ++t) {
-            const int jt = sh_j[t];
-            const T *rec = sh_r[t];
-            T gj[NLM][NP];
+            const float *row = io.gA + (size_t)sm.j[t] * NLM * C + co;
+            T b[KY];
+            ld_rec<KY / V4>(sm.rec[t], b);
+            T wl[NL][NP];
 #pragma unroll
-            for (int lm = 0; lm < NLM; ++lm) ldp<CPW>(io.gA + ((size_t)jt * NLM + lm) * C + lane * CPW, gj[lm]);
+            for (int lm = 0; lm < NLM; ++lm) {
+                const int l = lm == 0 ? 0 : (lm < 4 ? 1 : 2);
+                T gj[NP];
+                ldp<CPW>(row + lm * C, gj);
 #pragma unroll
-            for (int p = 0; p < NP; ++p) {
+                for (int p = 0; p < NP; ++p)
+                    wl[l][p] = lm == l * l ? vmul(gj[p], b[K + lm]) : vfma(gj[p], b[K + lm], wl[l][p]);
+            }
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
 #pragma unroll
                 for (int l = 0; l < NL; ++l) {
-                    T s0 = vdup<T>(0.f), s2 = vdup<T>(0.f);
+                    T s0 = vmul(W[l][0][p], b[0]), s2 = vmul(W[l][1][p], b[1]);
 #pragma unroll
-                    for (int k = 0; k < K; k += 2) {
-                        s0 = vfma(W[l][k][p], rec[k], s0);
-                        s2 = vfma(W[l][k + 1][p], rec[k + 1], s2);
+                    for (int k = 2; k < K; k += 2) {
+                        s0 = vfma(W[l][k][p], b[k], s0);
+                        s2 = vfma(W[l][k + 1][p], b[k + 1], s2);
                     }
                     const T R = vadd(s0, s2);
-                    T wl = vdup<T>(0.f);
-#pragma unroll
-                    for (int lm = l * l; lm < (l + 1) * (l + 1); ++lm) wl = vfma(gj[lm][p], rec[2 * K + lm], wl);
-                    if (l & 1) gso[p] = vfma(R, wl, gso[p]);
-                    else gse[p] = vfma(R, wl, gse[p]);
+                    if (l & 1) gso[p] = vfma(R, wl[l][p], gso[p]);
+                    else gse[p] = vfma(R, wl[l][p], gse[p]);
                 }
-            }
         }
-        for (int t0 = n_lo; t0 < n_lo + n_up; t0 += FT) {
-            const int t1 = min(n_lo + n_up, t0 + FT);
-#pragma unroll 2
-            for (int t = t0; t < t1; ++t) {
-                const int jt = sh_j[t];
-                const T *rec = sh_r[t];
-                const float *ge = sh_g[t];
-                T sj[NP];
-                ldp<CPW>(io.s + (size_t)jt * C + lane * CPW, sj);
-                T gj[NLM][NP];
+#pragma unroll 1   // (two pairs at a time: 779 us, the compiler runs out of registers)
+        for (int t = n_lo; t < nt; ++t) {
+            const int jt = sm.j[t];
+            const float *row = io.gA + (size_t)jt * NLM * C + co;
+            T b[KY + K];
+            ld_rec<(KY + K) / V4>(sm.rec[t], b);
+            T sj[NP], rho, beta[NLM];
+            ldp<CPW>(io.s + (size_t)jt * C + co, sj);
+            rho = vdup<T>(0.f);
+            T R[NL][NP], Rp[NL][NP];
 #pragma unroll
-                for (int lm = 0; lm < NLM; ++lm) ldp<CPW>(io.gA + ((size_t)jt * NLM + lm) * C + lane * CPW, gj[lm]);
-                T y[NLM];
+            for (int p = 0; p < NP; ++p)
 #pragma unroll
-                for (int lm = 0; lm < NLM; ++lm) y[lm] = rec[2 * K + lm];
-                T rho = vdup<T>(0.f), beta[NLM];
+                for (int l = 0; l < NL; ++l) {
+                    T s0 = vmul(W[l][0][p], b[0]), s1 = vmul(W[l][0][p], b[KY]), s2 = vmul(W[l][1][p], b[1]),
+                      s3 = vmul(W[l][1][p], b[KY + 1]);
 #pragma unroll
-                for (int lm = 0; lm < NLM; ++lm) beta[lm] = vdup<T>(0.f);
+                    for (int k = 2; k < K; k += 2) {
+                        s0 = vfma(W[l][k][p], b[k], s0);
+                        s1 = vfma(W[l][k][p], b[KY + k], s1);
+                        s2 = vfma(W[l][k + 1][p], b[k + 1], s2);
+                        s3 = vfma(W[l][k + 1][p], b[KY + k + 1], s3);
+                    }
+                    R[l][p] = vadd(s0, s2);
+                    Rp[l][p] = vadd(s1, s3);
+                }
+#pragma unroll
+            for (int l = 0; l < NL; ++l) {
+                T tl[NP], wl[NP];
+#pragma unroll
+                for (int lm = l * l; lm < (l + 1) * (l + 1); ++lm) {
+                    T gj[NP], ga[NP];
+                    ldp<CPW>(row + lm * C, gj);
+                    ldp_s<CPW>(sm.ga + lm * C + co, ga);
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) {
+                        const T gam = vfma(ga[p], sj[p], vmul(gj[p], (l & 1) ? san[p] : sa[p]));
+                        const T y = b[K + lm];
+                        tl[p] = lm == l * l ? vmul(gam, y) : vfma(gam, y, tl[p]);
+                        beta[lm] = p == 0 ? vmul(gam, R[l][p]) : vfma(gam, R[l][p], beta[lm]);
+                        wl[p] = lm == l * l ? vmul(gj[p], y) : vfma(gj[p], y, wl[p]);
+                    }
+                }
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
-                    T R[NL], Rp[NL];
-#pragma unroll
-                    for (int l = 0; l < NL; ++l) {
-                        T s0 = vdup<T>(0.f), s1 = vdup<T>(0.f), s2 = vdup<T>(0.f), s3 = vdup<T>(0.f);
-#pragma unroll
-                        for (int k = 0; k < K; k += 2) {
-                            s0 = vfma(W[l][k][p], rec[k], s0);
-                            s1 = vfma(W[l][k][p], rec[K + k], s1);
-                            s2 = vfma(W[l][k + 1][p], rec[k + 1], s2);
-                            s3 = vfma(W[l][k + 1][p], rec[K + k + 1], s3);
-                        }
-                        R[l] = vadd(s0, s2);
-                        Rp[l] = vadd(s1, s3);
-                    }
-#pragma unroll
-                    for (int l = 0; l < NL; ++l) {
-                        const T sas = (l & 1) ? san[p] : sa[p];
-                        T tl = vdup<T>(0.f), wl = vdup<T>(0.f);
-#pragma unroll
-                        for (int lm = l * l; lm < (l + 1) * (l + 1); ++lm) {
-                            const T gam = vfma(sh_ga[lm][p * 32 + lane], sj[p], vmul(gj[lm][p], sas));
-                            tl = vfma(gam, y[lm], tl);
-                            beta[lm] = vfma(gam, R[l], beta[lm]);
-                            wl = vfma(gj[lm][p], y[lm], wl);
-                        }
-                        rho = vfma(Rp[l], tl, rho);
-                        if (l & 1) gso[p] = vfma(R[l], wl, gso[p]);
-                        else gse[p] = vfma(R[l], wl, gse[p]);
-                    }
-                }
-                // this lane's share (its channels) of the pair's force on a
-                const float rh = vsum(rho);
-                float ex = rh * ge[3 * NLM], ey = rh * ge[3 * NLM + 1], ez = rh * ge[3 * NLM + 2];
-#pragma unroll
-                for (int lm = 1; lm < NLM; ++lm) {
-                    const float bl = vsum(beta[lm]);
-                    ex = fmaf(bl, ge[3 * lm], ex);
-                    ey = fmaf(bl, ge[3 * lm + 1], ey);
-                    ez = fmaf(bl, ge[3 * lm + 2], ez);
-                }
-                sh_f[0][t - t0][lane] = ex;
-                sh_f[1][t - t0][lane] = ey;
-                sh_f[2][t - t0][lane] = ez;
-            }
-            __syncwarp();
-            // pair t0 + u: lanes u and u + 16 add up lanes 0-15 and 16-31 of
-            // its shares (conflict-free: row stride 33), then lane u the two
-            // halves, in a fixed order
-            const int u = lane & (FT - 1), h = lane / FT;
-            const bool own = t0 + u < t1;
-            float px = 0.f, py = 0.f, pz = 0.f;
-            if (own) {
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    px += sh_f[0][u][16 * h + q];
-                    py += sh_f[1][u][16 * h + q];
-                    pz += sh_f[2][u][16 * h + q];
+                    rho = vfma(Rp[l][p], tl[p], rho);
+                    if (l & 1) gso[p] = vfma(R[l][p], wl[p], gso[p]);
+                    else gse[p] = vfma(R[l][p], wl[p], gse[p]);
                 }
             }
-            px += __shfl_down_sync(DMTS_FULL, px, 16);
-            py += __shfl_down_sync(DMTS_FULL, py, 16);
-            pz += __shfl_down_sync(DMTS_FULL, pz, 16);
-            if (own && h == 0) {
-                const int jt = sh_j[t0 + u];
-                px *= io.nu;
-                py *= io.nu;
-                pz *= io.nu;
-                if (fix_ok(px) && fix_ok(py) && fix_ok(pz)) {
-                    const long long qx = to_fix(px), qy = to_fix(py), qz = to_fix(pz);
-                    oa[0] += qx;
-                    oa[1] += qy;
-                    oa[2] += qz;
-                    unsigned long long *fj = io.Ffix + 3 * (size_t)jt;
-                    fix_add(fj, -qx);
-                    fix_add(fj + 1, -qy);
-                    fix_add(fj + 2, -qz);
-                    if (VIR) {
-                        // virial proxy: dU/dd . d of the pair, half to each end
-                        const float *ge = sh_g[t0 + u];
-                        const float wp = 0.5f * ge[3 * NLM + 3] * (px * ge[3 * NLM] + py * ge[3 * NLM + 1] + pz * ge[3 * NLM + 2]);
-                        if (fix_ok(wp)) {
-                            const long long qw = to_fix(wp);
-                            ow += qw;
-                            fix_add(io.Wfix + jt, qw);
-                        } else {
-                            bad = true;
-                        }
-                    }
-                } else {
-                    bad = true;
+            // this lane's share (its channels) of the pair's force on a:
+            // dY_lm/dd = (G_lm - (G_lm . n) n) / r with G_lm = grad_n Y_lm
+            const float4 n = sm.dir[t];
+            float h = vsum(rho), ex = 0.f, ey = 0.f, ez = 0.f;
+            if (LMAX >= 1) {
+                const float s3 = 1.7320508075688772f;
+                float gx = s3 * vsum(beta[LMAX >= 1 ? 1 : 0]), gy = s3 * vsum(beta[LMAX >= 1 ? 2 : 0]),
+                      gz = s3 * vsum(beta[LMAX >= 1 ? 3 : 0]);
+                if (LMAX >= 2) {
+                    const float s15 = 3.872983346207417f, s5 = 2.23606797749979f;
+                    const float b4 = s15 * vsum(beta[LMAX >= 2 ? 4 : 0]), b5 = s15 * vsum(beta[LMAX >= 2 ? 5 : 0]),
+                                b6 = 3.f * s5 * vsum(beta[LMAX >= 2 ? 6 : 0]),
+                                b7 = s15 * vsum(beta[LMAX >= 2 ? 7 : 0]), b8 = s15 * vsum(beta[LMAX >= 2 ? 8 : 0]);
+                    gx = fmaf(n.y, b4, fmaf(n.z, b7, fmaf(n.x, b8, gx)));
+                    gy = fmaf(n.x, b4, fmaf(n.z, b5, fmaf(-n.y, b8, gy)));
+                    gz = fmaf(n.y, b5, fmaf(n.x, b7, fmaf(n.z, b6, gz)));
                 }
+                h = fmaf(-n.w, fmaf(gx, n.x, fmaf(gy, n.y, gz * n.z)), h);
+                ex = gx * n.w;
+                ey = gy * n.w;
+                ez = gz * n.w;
             }
-            __syncwarp();
+            const int u = (t - n_lo) & (FT - 1);
+            sm.f[0][u][lane] = fmaf(h, n.x, ex);
+            sm.f[1][u][lane] = fmaf(h, n.y, ey);
+            sm.f[2][u][lane] = fmaf(h, n.z, ez);
+            const int done = t + 1 - n_lo;
+            if (((done & (FT - 1)) == 0 || t + 1 == nt)) {
+                __syncwarp();   // the shares are written
+                // pair t0 + u: lanes u, u + 8, .. add up eight lanes' shares each
+                // (conflict-free: row stride 33), then lane u the four parts, in
+                // a fixed order
+                const int t0 = n_lo + ((done - 1) & ~(FT - 1));
+                const int u = lane & (FT - 1), h = lane / FT;
+                const bool own = t0 + u <= t;
+                float px = 0.f, py = 0.f, pz = 0.f;
+                if (own) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        px += sm.f[0][u][8 * h + q];
+                        py += sm.f[1][u][8 * h + q];
+                        pz += sm.f[2][u][8 * h + q];
+                    }
+                }
+                px += __shfl_down_sync(DMTS_FULL, px, 16);
+                py += __shfl_down_sync(DMTS_FULL, py, 16);
+                pz += __shfl_down_sync(DMTS_FULL, pz, 16);
+                px += __shfl_down_sync(DMTS_FULL, px, 8);
+                py += __shfl_down_sync(DMTS_FULL, py, 8);
+                pz += __shfl_down_sync(DMTS_FULL, pz, 8);
+                if (own && h == 0) {
+                    const int jt = sm.j[t0 + u];
+                    px *= io.nu;
+                    py *= io.nu;
+                    pz *= io.nu;
+                    if (fix_ok(px) && fix_ok(py) && fix_ok(pz)) {
+                        const long long qx = to_fix(px), qy = to_fix(py), qz = to_fix(pz);
+                        oa[0] += qx;
+                        oa[1] += qy;
+                        oa[2] += qz;
+                        unsigned long long *fj = io.Ffix + 3 * (size_t)jt;
+                        fix_add(fj, -qx);
+                        fix_add(fj + 1, -qy);
+                        fix_add(fj + 2, -qz);
+                        if (VIR) {
+                            // virial proxy: dU/dd . d of the pair, half to each end
+                            const float4 n = sm.dir[t0 + u];
+                            const float wv = 0.5f / n.w * (px * n.x + py * n.y + pz * n.z);
+                            if (fix_ok(wv)) {
+                                const long long qw = to_fix(wv);
+                                ow += qw;
+                                fix_add(io.Wfix + jt, qw);
+                            } else {
+                                bad = true;
+                            }
+                        }
+                    } else {
+                        bad = true;
+                    }
+                }
+                __syncwarp();
+            }
         }
         __syncwarp();
     }
@@ -445,16 +489,16 @@ __global__ void __launch_bounds__(BWD_WARPS * 32) k_mp_bwd(EdgeGeom g, LayerIO i
         if (VIR) fix_add(io.Wfix + a, ow);
     }
     T gin[NP], gout[NP];
-    ldp<CPW>(io.gs_in + (size_t)a * C + lane * CPW, gin);
+    ldp<CPW>(io.gs_in + (size_t)a * C + co, gin);
 #pragma unroll
     for (int p = 0; p < NP; ++p) gout[p] = vfma(vdup<T>(io.nu), vsub(gse[p], gso[p]), gin[p]);
-    stp<CPW>(io.gs_out + (size_t)a * C + lane * CPW, gout);
+    stp<CPW>(io.gs_out + (size_t)a * C + co, gout);
     if (io.gs_out_bf16) {
 #pragma unroll
         for (int p = 0; p < NP; ++p)
 #pragma unroll
             for (int hh = 0; hh < PW; ++hh)
-                st_split(io.gs_out_bf16, a, C, lane * CPW + p * PW + hh, vget(gout[p], hh));
+                st_split(io.gs_out_bf16, a, C, co + p * PW + hh, vget(gout[p], hh));
     }
 }
 
@@ -496,11 +540,9 @@ static void fwd_c(const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
 
 template <int C, int LMAX, bool VIR>
 static void bwd_launch(const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
-    constexpr size_t smem = BwdSmem<C, LMAX, 8, VIR>::bytes;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_mp_bwd<C, LMAX, 8, VIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int blocks = (g.n_atoms + BWD_WARPS - 1) / BWD_WARPS;
-    k_mp_bwd<C, LMAX, 8, VIR><<<blocks, BWD_WARPS * 32, smem, st>>>(g, io);
+    constexpr size_t smem = sizeof(BwdSmem<C, LMAX, 8>);
+    static_assert(smem <= 48 * 1024, "shared memory without an opt-in");
+    k_mp_bwd<C, LMAX, 8, VIR><<<g.n_atoms, 32, smem, st>>>(g, io);
     count_launch();
 }
 
