@@ -281,8 +281,9 @@ static FirstIO first_io(dmts_ctx *ctx, const SysView &s, const DevModel &m) {
 // One node-level contraction: the tensor cores (split-bf16 operands) for a
 // model that runs its MLPs in bf16, whatever the number of rows M (a batch
 // smaller than one 128-row tile reads zero-filled rows), so that an atom's
-// arithmetic never depends on the batch it is in; the fp32 SIMT kernel for
-// an fp32 model. trans/W32 describe the fp32 weight, Wt16 the K-major
+// arithmetic never depends on the batch it is in; for an fp32 model the
+// tensor cores with operands in three parts from 128 channels on, below them
+// the fp32 SIMT kernel. trans/W32 describe the fp32 weight, Wt16 the K-major
 // split-bf16 copy. False (with the context's error text set) when a bf16
 // model's contraction cannot be launched.
 static bool contract(dmts_ctx *ctx, const DevModel &m, int M, int N, int K, const float *A32,
@@ -295,7 +296,10 @@ static bool contract(dmts_ctx *ctx, const DevModel &m, int M, int N, int K, cons
         return false;
     }
     ProfScope ps(ctx, tag_f32, st);
-    launch_gemm_f32(M, N, K, A32, W32, trans, e, st);
+    // (23,558 rows, C = 128: the 14 contractions of a conservative call 777 us
+    // SIMT, 510 split; at 192 rows of C = 64 7.4 us a call SIMT, 11.1 split)
+    if (std::min(N, K) >= 128) launch_gemm_split(M, N, K, A32, W32, trans, e, ctx->d_err, st);
+    else launch_gemm_f32(M, N, K, A32, W32, trans, e, st);
     return true;
 }
 
@@ -1137,15 +1141,21 @@ dmts_status nc_distill_step(dmts_ctx *ctx, const dmts_system *sys, const dmts_nb
     const float *s1 = (const float *)w.nc_s.p + (size_t)N * C;
     float *part_buf = (float *)w.dist_part.p;
     if (fit_qk) launch_atb(N, QKW, C, gqk, s1, at(m.Wqk), nullptr, part_buf, st);   // dW_qk = gQK^T s1
+    // Gradients are sums over the batch: here the split contractions go by the
+    // number of rows (49,152 rows, C = 64: 100 us SIMT for the three, 60 split)
+    auto gemm = [&](int M, int Nc, int K, const float *A, const float *W, int trans, const Epi &e) {
+        if (M >= 8192 && std::min(Nc, K) >= 64) launch_gemm_split(M, Nc, K, A, W, trans, e, ctx->d_err, st);
+        else launch_gemm_f32(M, Nc, K, A, W, trans, e, st);
+    };
     if (fit_mlp || fit_layer) {
         // s1 = s0 + act W2^T + b2, act = silu(h), h = q W1^T + b1
         Epi e = epi(EPI_STORE);
         e.out = gs1;
-        launch_gemm_f32(N, C, QKW, gqk, m.Wqk, 0, e, st);                               // g_s1 = gQK W_qk
+        gemm(N, C, QKW, gqk, m.Wqk, 0, e);   // g_s1 = gQK W_qk
         Epi ed = epi(EPI_DSILU);
         ed.H = (float *)w.dist_h.p;
         ed.out = gh;
-        launch_gemm_f32(N, C, C, gs1, m.w2[0], 0, ed, st);                             // g_h = (g_s1 W2) silu'(h)
+        gemm(N, C, C, gs1, m.w2[0], 0, ed);   // g_h = (g_s1 W2) silu'(h)
         if (fit_mlp) {
             launch_atb(N, C, C, gs1, (const float *)w.nc_act.p, at(m.w2[0]), at(m.b2[0]), part_buf, st);
             launch_atb(N, C, 2 * C, gh, (const float *)w.nc_q.p, at(m.w1[0]), at(m.b1[0]), part_buf, st);
@@ -1155,7 +1165,7 @@ dmts_status nc_distill_step(dmts_ctx *ctx, const dmts_system *sys, const dmts_nb
         // q = (A_00^2, sum_m A_1m^2) per channel, V_t = sum_c U[t][c] A_1m[c]
         Epi e = epi(EPI_STORE);
         e.out = (float *)w.dist_gq.p;
-        launch_gemm_f32(N, 2 * C, C, gh, m.w1[0], 0, e, st);                           // g_q = g_h W1
+        gemm(N, 2 * C, C, gh, m.w1[0], 0, e);   // g_q = g_h W1
         NCLayerGradArgs la;
         la.n_atoms = N;
         la.nu = m.nu;

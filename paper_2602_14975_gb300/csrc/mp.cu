@@ -566,7 +566,8 @@ void launch_mp_bwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io,
 }
 
 // -------------------------------------------------------------------- GEMM
-// fp32 SIMT contraction. A CTA computes a BM x BN tile; K is walked in chunks
+// fp32 SIMT contraction (fp32 models of fewer than 128 channels, small
+// gradients; the others: gemm_split.cu). A CTA computes a BM x BN tile; K is walked in chunks
 // of 32, GEMM_STAGES of them in flight (16-byte asynchronous copies, zero
 // filled past M, N and K). Both tiles are kept k-contiguous (row stride 36:
 // the eight rows a quarter-warp reads with 16-byte loads lie in distinct

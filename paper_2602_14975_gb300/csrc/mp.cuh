@@ -153,6 +153,9 @@ struct Epi {
 // or W for W [K][N] (trans = 0); fp32 SIMT.
 void launch_gemm_f32(int M, int N, int K, const float *Act, const float *W, int trans, const Epi &e,
                      cudaStream_t st);
+// The same on the tensor cores, operands in three bf16 parts (24 bits).
+void launch_gemm_split(int M, int N, int K, const float *Act, const float *W, int trans, const Epi &e, int *err,
+                       cudaStream_t st);
 // Out[M][N] = Act[M][K] x Wt^T on the tensor cores (tcgen05, bf16 operands,
 // fp32 accumulator in tensor memory), Wt K-major [N][K]. With split = 1 both
 // operands are split-bf16 copies (rows of 2K: hi | lo, common.cuh) and
