@@ -658,19 +658,17 @@ SysView state_view(dmts_state *stt) {
 void rebuild_lists(dmts_ctx *ctx, StateInternal *si, const SysView &v, cudaStream_t st) {
     NbrWork nw;
     prepare_nbr_work_async(ctx, si, v, nw);
-    { ProfScope ps(ctx, "nbr_cells", st); nbr_cells(nw, si->r_cons, st); }
-    {
-        // the full list and, in the same pass, the NC list within r_nc + skin
-        ProfScope ps(ctx, "nbr_fill", st);
-        if (ctx->has_nc)
-            nbr_fill(nw, si->r_cons, (int *)si->cons_row.p, (int *)si->cons_col.p, si->cons_cap, (float *)si->x_ref.p,
-                     st, si->r_nc, (int *)si->nc_row.p, (int *)si->nc_col.p, si->nc_cap);
-        else
-            nbr_fill(nw, si->r_cons, (int *)si->cons_row.p, (int *)si->cons_col.p, si->cons_cap, (float *)si->x_ref.p,
-                     st);
+    if (v.n == 0) {
+        k_set_int<<<1, 1, 0, st>>>((int *)si->gate.p, 0);
+        count_launch();
+        return;
     }
-    k_set_int<<<1, 1, 0, st>>>((int *)si->gate.p, 0);
-    count_launch();
+    // the full list and, in the same pass, the NC list within r_nc + skin
+    ProfScope ps(ctx, "nbr_rebuild", st);
+    const bool nc = ctx->has_nc;
+    nbr_rebuild(nw, si->r_cons, (int *)si->cons_row.p, (int *)si->cons_col.p, si->cons_cap, (float *)si->x_ref.p,
+                (unsigned *)si->scratch.sync.p, (int *)si->gate.p, st, nc ? si->r_nc : 0.f,
+                nc ? (int *)si->nc_row.p : nullptr, nc ? (int *)si->nc_col.p : nullptr, nc ? si->nc_cap : -1);
 }
 
 void prepare_nbr_work_async(dmts_ctx *ctx, StateInternal *si, const SysView &v, NbrWork &nw) {
@@ -837,7 +835,8 @@ dmts_status init_state(dmts_ctx *ctx, dmts_state *stt, float skin, cudaStream_t 
     const double frac = ctx->has_nc ? std::pow(si->r_nc / si->r_cons, 3.0) : 0.0;
     const long long want_nc = (long long)(tot * frac * 1.6) + 16LL * N + 1024;
     if (!si->cons_col.ensure(sizeof(int) * want_cons) || !si->nc_col.ensure(sizeof(int) * want_nc) ||
-        !si->scratch.slots.ensure(sizeof(int) * (size_t)N * kNbrSlots))
+        !si->scratch.slots.ensure(sizeof(int) * (size_t)N * kNbrSlots) ||
+        !ensure_zeroed(ctx, si->scratch.sync, sizeof(unsigned) * (2 + kRebuildBlocks), st))
         return fail(ctx, DMTS_E_OOM, "neighbour list allocation failed");
     si->cons_cap = (long long)(si->cons_col.cap / sizeof(int));
     si->nc_cap = (long long)(si->nc_col.cap / sizeof(int));

@@ -59,11 +59,12 @@ struct NbrScratch {
     Buf grid, cell_cnt, cell_start, cell_atoms, atom_cell, atom_slot, counts, total, counts_sub;
     Buf slots;    // [n_atoms][kNbrSlots] sorted rows kept between the count and the fill
     Buf scan;     // prefix-scan status words [2][scan_tiles] and epoch/tile counters [2] (zero-initialised)
+    Buf sync;     // barrier words of a state's rebuild (zero-initialised)
     int scan_tiles = 0;
     void release_all() {
         grid.release(); cell_cnt.release(); cell_start.release(); cell_atoms.release();
         atom_cell.release(); atom_slot.release(); counts.release(); total.release(); counts_sub.release();
-        slots.release(); scan.release();
+        slots.release(); scan.release(); sync.release();
         scan_tiles = 0;
     }
 };

@@ -2,6 +2,8 @@
 // replicas). Cell grids have edge >= r_list, so all pairs lie in the 27 (or
 // fewer, de-duplicated) neighbouring cells. Rows are sorted by neighbour
 // index, so their order is canonical and independent of scheduling.
+#include <algorithm>
+
 #include "nbr.cuh"
 #include "ptx.cuh"
 
@@ -24,9 +26,7 @@ void atom_rep_map(const int *rep_off, int n_rep, int n_atoms, int *atom_rep, cud
 
 // One block per replica: zeroes the replica's cell counts; open replicas:
 // bounding box -> origin and cell edge max(r_list, extent/dim).
-__global__ void k_grid_open(NbrWork w, float r_list) {
-    if (gated_off(w.gate, w.err)) return;
-    const int r = blockIdx.x;
+__device__ __forceinline__ void grid_open(const NbrWork &w, float r_list, int r) {
     CellGrid &g = w.grid[r];
     const int nc = g.dim[0] * g.dim[1] * g.dim[2];
     for (int c = threadIdx.x; c < nc; c += blockDim.x) w.cell_cnt[g.cell_off + c] = 0;
@@ -71,6 +71,9 @@ __global__ void k_grid_open(NbrWork w, float r_list) {
         }
     }
 }
+__global__ void k_grid_open(NbrWork w, float r_list) {
+    if (!gated_off(w.gate, w.err)) grid_open(w, r_list, blockIdx.x);
+}
 
 __device__ __forceinline__ int cell_coord(float v, const CellGrid &g, int a) {
     int c;
@@ -83,10 +86,7 @@ __device__ __forceinline__ int cell_coord(float v, const CellGrid &g, int a) {
     return min(max(c, 0), g.dim[a] - 1);
 }
 
-__global__ void k_cell_assign(NbrWork w) {
-    if (gated_off(w.gate, w.err)) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= w.n_atoms) return;
+__device__ __forceinline__ void cell_assign(const NbrWork &w, int i) {
     const CellGrid g = w.grid[w.atom_rep[i]];
     const int cx = cell_coord(w.x[3 * i], g, 0), cy = cell_coord(w.x[3 * i + 1], g, 1),
               cz = cell_coord(w.x[3 * i + 2], g, 2);
@@ -94,12 +94,17 @@ __global__ void k_cell_assign(NbrWork w) {
     w.atom_cell[i] = cell;
     w.atom_slot[i] = atomicAdd(&w.cell_cnt[cell], 1);
 }
-
-__global__ void k_cell_scatter(NbrWork w) {
-    if (gated_off(w.gate, w.err)) return;
+__global__ void k_cell_assign(NbrWork w) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= w.n_atoms) return;
+    if (i < w.n_atoms && !gated_off(w.gate, w.err)) cell_assign(w, i);
+}
+
+__device__ __forceinline__ void cell_scatter(const NbrWork &w, int i) {
     w.cell_atoms[w.cell_start[w.atom_cell[i]] + w.atom_slot[i]] = i;
+}
+__global__ void k_cell_scatter(NbrWork w) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < w.n_atoms && !gated_off(w.gate, w.err)) cell_scatter(w, i);
 }
 
 // Visits every candidate j of atom i (fixed cell order, ascending j inside a
@@ -353,13 +358,17 @@ struct RowAcc {
 // per-atom sweep; a cell with more candidates than fit falls back to it.
 constexpr int NBC_WARPS = 8, NBC_CAP = 2048;
 
-__global__ void __launch_bounds__(NBC_WARPS * 32) k_nbr_count_cell(NbrWork w, float rc2, float rc2_sub) {
-    if (gated_off(w.gate, w.err)) return;
-    __shared__ int cj[NBC_CAP];
-    __shared__ float cx[NBC_CAP], cy[NBC_CAP], cz[NBC_CAP];
-    __shared__ __align__(16) int buf[NBC_WARPS][NB_MAXROW];
-    __shared__ int seg_beg[18], seg_excl[19];
-    const int c = blockIdx.x;
+struct CountSmem {
+    int cj[NBC_CAP];
+    float cx[NBC_CAP], cy[NBC_CAP], cz[NBC_CAP];
+    alignas(16) int buf[NBC_WARPS][NB_MAXROW];
+    int seg_beg[18], seg_excl[19];
+};
+
+__device__ __forceinline__ void count_cell(const NbrWork &w, float rc2, float rc2_sub, int c, CountSmem &sm) {
+    int *cj = sm.cj, *seg_beg = sm.seg_beg, *seg_excl = sm.seg_excl;
+    float *cx = sm.cx, *cy = sm.cy, *cz = sm.cz;
+    int (*buf)[NB_MAXROW] = sm.buf;
     const int a_beg = w.cell_start[c], a_end = w.cell_start[c + 1];
     if (a_beg == a_end) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -452,6 +461,10 @@ __global__ void __launch_bounds__(NBC_WARPS * 32) k_nbr_count_cell(NbrWork w, fl
         acc.finish(w, keep, i, lane);
     }
 }
+__global__ void __launch_bounds__(NBC_WARPS * 32) k_nbr_count_cell(NbrWork w, float rc2, float rc2_sub) {
+    __shared__ CountSmem sm;
+    if (!gated_off(w.gate, w.err)) count_cell(w, rc2, rc2_sub, blockIdx.x, sm);
+}
 
 // Appends, in order, the entries of the sorted row src[0..n) within rc2_sub
 // to dst (warp-cooperative; distances recomputed exactly as in the build).
@@ -479,15 +492,9 @@ __device__ __forceinline__ void write_sub_row(const NbrWork &w, int i, const int
     }
 }
 
-__global__ void __launch_bounds__(NB_WARPS * 32) k_nbr_fill_warp(NbrWork w, float rc2, const int *row_ptr, int *col,
-                                                                 float *x_ref, float rc2_sub, const int *sub_row,
-                                                                 int *sub_col) {
-    if (gated_off(w.gate, w.err)) return;
-    __shared__ __align__(16) int buf[NB_WARPS][NB_MAXROW];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * NB_WARPS + warp;
-    if (i >= w.n_atoms) return;
-    int *sb = buf[warp];
+// Row i by one warp (sb: NB_MAXROW entries of its own).
+__device__ __forceinline__ void fill_row(const NbrWork &w, float rc2, const int *row_ptr, int *col, float *x_ref,
+                                         float rc2_sub, const int *sub_row, int *sub_col, int i, int *sb, int lane) {
     const int beg = row_ptr[i], n = row_ptr[i + 1] - beg;
     if (w.slots && n <= w.slot_cap && n <= NB_MAXROW) {
         // the count pass kept the sorted row: copy it, sub entries by their flag
@@ -539,6 +546,15 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_nbr_fill_warp(NbrWork w, floa
         x_ref[3 * i + 2] = w.x[3 * i + 2];
     }
 }
+__global__ void __launch_bounds__(NB_WARPS * 32) k_nbr_fill_warp(NbrWork w, float rc2, const int *row_ptr, int *col,
+                                                                 float *x_ref, float rc2_sub, const int *sub_row,
+                                                                 int *sub_col) {
+    if (gated_off(w.gate, w.err)) return;
+    __shared__ __align__(16) int buf[NB_WARPS][NB_MAXROW];
+    const int warp = threadIdx.x >> 5, i = blockIdx.x * NB_WARPS + warp;
+    if (i < w.n_atoms)
+        fill_row(w, rc2, row_ptr, col, x_ref, rc2_sub, sub_row, sub_col, i, buf[warp], threadIdx.x & 31);
+}
 
 // ------------------------------------------------------------ prefix scan
 // Decoupled look-back: each block takes the next tile in order (a counter,
@@ -563,18 +579,14 @@ struct ScanJob {
     long long *total;
 };
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan(ScanJob j0, ScanJob j1, int n, int n_tiles,
-                                                       unsigned long long *status_all, unsigned long long *counters,
-                                                       int tiles_cap, int *err, const int *gate) {
-    if (gated_off(gate, err)) return;
-    const ScanJob J = blockIdx.y ? j1 : j0;
-    unsigned long long *status = status_all + (size_t)blockIdx.y * tiles_cap;
-    unsigned long long *counter = counters + blockIdx.y;
+// The next tile of job J (block-wide).
+__device__ __forceinline__ void scan_tile(const ScanJob &J, int n, int n_tiles, unsigned long long *status,
+                                          unsigned long long *counter, int *err) {
     __shared__ int tile_sh;
     __shared__ unsigned tag_sh;
     __shared__ long long warp_tot[SCAN_THREADS / 32], excl_sh;
     if (threadIdx.x == 0) {
-        // every block of this launch takes one tile and reads the same epoch;
+        // every tile of a scan is taken once and reads the same epoch;
         // the block that takes the last one opens the next epoch
         const unsigned long long old = atomicAdd(counter, 1ull);
         const int t = (int)(old & 0xffffffffull);
@@ -654,6 +666,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(ScanJob j0, ScanJob j1, i
     }
 }
 
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan(ScanJob j0, ScanJob j1, int n, int n_tiles,
+                                                       unsigned long long *status_all, unsigned long long *counters,
+                                                       int tiles_cap, int *err, const int *gate) {
+    if (gated_off(gate, err)) return;
+    scan_tile(blockIdx.y ? j1 : j0, n, n_tiles, status_all + (size_t)blockIdx.y * tiles_cap, counters + blockIdx.y, err);
+}
+
 void scan_ints(const NbrWork &w, const int *in0, int *out0, long long cap0, long long *total0, const int *in1,
                int *out1, long long cap1, long long *total1, int n, cudaStream_t st) {
     const int tiles = (n + kScanTile - 1) / kScanTile;
@@ -693,6 +712,155 @@ void nbr_fill(const NbrWork &w, float r_list, int *row_ptr, int *col, long long 
                                                       wc.counts_sub ? sub_col : nullptr);
         count_launch();
     }
+}
+
+// ----------------------------------------------------------- gated rebuild
+// A state's rebuild as one cooperative launch: the phases above with barriers
+// over the grid between them. Every inner step asks for one and most find the
+// gate closed; as eight launches (cells, scans, count, fill, gate) that cost
+// XX.
+//
+// Barrier: block b > 0 writes the epoch (launch number, phase) to its word and
+// waits for block 0's release word; block 0 collects the words, reads the
+// error word once for everybody and releases with a stop bit. Every wait is
+// bounded; words of an earlier launch never match.
+constexpr int RB_THREADS = NBC_WARPS * 32;
+static_assert(RB_THREADS == SCAN_THREADS, "one block shape for every phase");
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// False: a stop (error recorded, or a block that never came).
+__device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned epoch, int *err) {
+    __shared__ int go;
+    unsigned *release = sync + 1, *words = sync + 2;
+    __syncthreads();
+    if (blockIdx.x == 0) {
+        int ok = 1;
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+            const uint64_t t0 = globaltimer_ns();
+            while (b > 0 && ok && ld_acquire(words + b) != epoch)
+                if (globaltimer_ns() - t0 > kWaitLimitNs) ok = 0;
+        }
+        ok = __syncthreads_and(ok);
+        if (threadIdx.x == 0) {
+            if (!ok) set_error(err, DMTS_E_TIMEOUT);
+            __threadfence();
+            go = ok && *(volatile int *)err == 0;
+            st_release(release, epoch << 1 | (go ? 0u : 1u));
+        }
+    } else if (threadIdx.x == 0) {
+        __threadfence();
+        st_release(words + blockIdx.x, epoch);
+        const uint64_t t0 = globaltimer_ns();
+        unsigned v;
+        bool ok = true;
+        while (((v = ld_acquire(release)) >> 1) != epoch && ok)
+            if (globaltimer_ns() - t0 > 2 * kWaitLimitNs) ok = false;
+        if (!ok) set_error(err, DMTS_E_TIMEOUT);
+        go = ok && !(v & 1u);
+        __threadfence();
+    }
+    __syncthreads();
+    return go != 0;
+}
+
+struct RebuildArgs {
+    float r_list, r_sub;
+    int *row_ptr, *col;
+    long long cap;
+    float *x_ref;
+    int *sub_row, *sub_col;
+    long long sub_cap;
+    int *gate;
+    unsigned *sync;   // launch number, release word, a word per block
+};
+
+__device__ __forceinline__ bool rebuild_phases(const NbrWork &w, const RebuildArgs &a, unsigned epoch, CountSmem &sm) {
+    const int tid = blockIdx.x * RB_THREADS + threadIdx.x, nthr = gridDim.x * RB_THREADS;
+    const float rc2 = a.r_list * a.r_list, rs2 = a.r_sub * a.r_sub;
+    auto scan = [&](const ScanJob &j0, const ScanJob &j1, int jobs, int n) {
+        const int tiles = max((n + kScanTile - 1) / kScanTile, 1);
+        for (int t = blockIdx.x; t < jobs * tiles; t += gridDim.x) {
+            const int y = t / tiles;
+            scan_tile(y ? j1 : j0, n, tiles, w.scan_status + (size_t)y * w.scan_tiles, w.scan_counter + y, w.err);
+            __syncthreads();
+        }
+    };
+    for (int r = blockIdx.x; r < w.n_rep; r += gridDim.x) {
+        grid_open(w, a.r_list, r);
+        __syncthreads();
+    }
+    if (!grid_barrier(a.sync, epoch, w.err)) return false;
+    for (int i = tid; i < w.n_atoms; i += nthr) cell_assign(w, i);
+    if (!grid_barrier(a.sync, epoch + 1, w.err)) return false;
+    const ScanJob cells{w.cell_cnt, w.cell_start, -1, nullptr};
+    scan(cells, cells, 1, w.n_cells);
+    if (!grid_barrier(a.sync, epoch + 2, w.err)) return false;
+    for (int i = tid; i < w.n_atoms; i += nthr) cell_scatter(w, i);
+    if (!grid_barrier(a.sync, epoch + 3, w.err)) return false;
+    for (int c = blockIdx.x; c < w.n_cells; c += gridDim.x) {
+        count_cell(w, rc2, rs2, c, sm);
+        __syncthreads();
+    }
+    if (!grid_barrier(a.sync, epoch + 4, w.err)) return false;
+    scan(ScanJob{w.counts, a.row_ptr, a.cap, w.total}, ScanJob{w.counts_sub, a.sub_row, a.sub_cap, nullptr},
+         w.counts_sub ? 2 : 1, w.n_atoms);
+    if (!grid_barrier(a.sync, epoch + 5, w.err)) return false;
+    const int warp = threadIdx.x >> 5;
+    for (int i = blockIdx.x * NBC_WARPS + warp; i < w.n_atoms; i += gridDim.x * NBC_WARPS) {
+        fill_row(w, rc2, a.row_ptr, a.col, a.x_ref, rs2, w.counts_sub ? a.sub_row : nullptr,
+                 w.counts_sub ? a.sub_col : nullptr, i, sm.buf[warp], threadIdx.x & 31);
+        __syncwarp();
+    }
+    return true;
+}
+
+__global__ void __launch_bounds__(RB_THREADS) k_nbr_rebuild(NbrWork w, RebuildArgs a) {
+    __shared__ CountSmem sm;
+    if (*(volatile int *)a.gate == 0) return;
+    const unsigned launch = *(volatile unsigned *)a.sync;
+    rebuild_phases(w, a, ((launch + 1) * 8u) & 0x7fffffffu, sm);   // (never the words' initial zero on the first)
+    // every other block is past its reads of both (the first barrier)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *a.gate = 0;
+        *a.sync = launch + 1;
+    }
+}
+
+void nbr_rebuild(const NbrWork &w, float r_list, int *row_ptr, int *col, long long capacity, float *x_ref,
+                 unsigned *sync, int *gate, cudaStream_t st, float r_sub, int *sub_row, int *sub_col,
+                 long long sub_capacity) {
+    static int fit = 0;
+    if (!fit) {
+        int dev = 0, n_sm = 1, per_sm = 1;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nbr_rebuild, RB_THREADS, 0);
+        fit = std::max(1, std::min(n_sm * per_sm, kRebuildBlocks));
+    }
+    NbrWork wc = w;
+    wc.gate = nullptr;
+    if (!sub_row) wc.counts_sub = nullptr;
+    RebuildArgs a{r_list, r_sub, row_ptr, col, capacity, x_ref, sub_row, sub_col, sub_capacity, gate, sync};
+    cudaLaunchConfig_t cfg = {};
+    // no more blocks than a phase has work for
+    cfg.gridDim = dim3(std::max(1, std::min(fit, std::max(w.n_cells, (w.n_atoms + NBC_WARPS - 1) / NBC_WARPS))));
+    cfg.blockDim = dim3(RB_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_nbr_rebuild, wc, a);
+    count_launch();
 }
 
 }  // namespace dmts

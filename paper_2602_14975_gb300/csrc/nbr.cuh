@@ -62,6 +62,13 @@ void nbr_cells(const NbrWork &w, float r_list, cudaStream_t st);
 void nbr_fill(const NbrWork &w, float r_list, int *row_ptr, int *col, long long capacity,
               float *x_ref, cudaStream_t st, float r_sub = 0.f, int *sub_row = nullptr, int *sub_col = nullptr,
               long long sub_capacity = -1);
+// The same, cells included, as one cooperative launch that does nothing while
+// *gate is 0 and clears it when done. sync: 2 + kRebuildBlocks words, zero when
+// allocated.
+constexpr int kRebuildBlocks = 1024;
+void nbr_rebuild(const NbrWork &w, float r_list, int *row_ptr, int *col, long long capacity, float *x_ref,
+                 unsigned *sync, int *gate, cudaStream_t st, float r_sub = 0.f, int *sub_row = nullptr,
+                 int *sub_col = nullptr, long long sub_capacity = -1);
 // Atom -> replica map.
 void atom_rep_map(const int *rep_off, int n_rep, int n_atoms, int *atom_rep, cudaStream_t st);
 // Exclusive scans of n ints into out[n+1], one or two arrays in one launch
