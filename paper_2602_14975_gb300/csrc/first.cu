@@ -24,6 +24,7 @@
 #include <algorithm>
 
 #include "edge.cuh"
+#include "launch.cuh"
 #include "mp.cuh"
 #include "pack.cuh"
 
@@ -107,6 +108,7 @@ struct FirstFwdSmem {
 // shared memory.
 template <int C, int LMAX>
 __global__ void __launch_bounds__((FirstFwdSmem<C, LMAX>::WARPS * 32), (FirstFwdSmem<C, LMAX>::CTAS)) k_first_fwd(EdgeGeom g, FirstIO io) {
+    dep_entry(g.n_atoms <= (int)(gridDim.x * (blockDim.x / 32)));
     using SM = FirstFwdSmem<C, LMAX>;
     constexpr int NL = SM::NL, NLM = SM::NLM, RS = SM::RS, TS = SM::TS, SLOTS = SM::SLOTS, WARPS = SM::WARPS;
     // channels in passes of 64 (two per lane): half the registers of one pass at C = 128
@@ -285,6 +287,7 @@ struct FirstBwdSmem {
 // lm, two species at a time) and one lane per edge for its force.
 template <int C, int LMAX, bool VIR>
 __global__ void __launch_bounds__(256, 2) k_first_bwd(EdgeGeom g, FirstIO io) {
+    dep_entry(g.n_atoms <= (int)(gridDim.x * (blockDim.x / 32)));
     using SM = FirstBwdSmem<C, LMAX>;
     constexpr int NL = SM::NL, NLM = SM::NLM, CPW = C / 32, WS = SM::WS, QS = SM::QS, WARPS = SM::WARPS;
     using T = typename Pack<CPW>::T;
@@ -466,7 +469,7 @@ void first_launch(Kern kern, int warps, size_t smem, const EdgeGeom &g, const Fi
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int fit = n_sm * resident_ctas(reinterpret_cast<const void *>(kern), warps * 32, smem, dev);
     const int grid = std::min((g.n_atoms + warps - 1) / warps, fit);
-    kern<<<grid, warps * 32, smem, st>>>(g, io);
+    launch_dep(kern, grid, warps * 32, smem, st, g, io);
     count_launch();
 }
 

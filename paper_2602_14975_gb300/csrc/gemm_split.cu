@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "epilogue.cuh"
+#include "launch.cuh"
 #include "mp.cuh"
 #include "ptx.cuh"
 #include "tc.cuh"
@@ -77,6 +78,7 @@ template <int BN, int ST, int TH, int MINB>
 __global__ void __launch_bounds__(TH, MINB) k_gemm_split(int M, int N, int K, const float *__restrict__ Act,
                                                                  const float *__restrict__ W, int trans, int vec, Epi e,
                                                                  int *err) {
+    dep_entry();
     using D = Gs<BN, ST, TH>;
     constexpr int CW = D::CW;
     extern __shared__ uint8_t gs_smem[];
@@ -237,7 +239,7 @@ static void gemm_split_launch(int M, int N, int K, const float *Act, const float
     constexpr uint32_t smem = Gs<BN, ST, TH>::SMEM;
     cudaFuncSetAttribute(k_gemm_split<BN, ST, TH, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     dim3 grid((N + BN - 1) / BN, (M + GS_BM - 1) / GS_BM);
-    k_gemm_split<BN, ST, TH, MINB><<<grid, TH, smem, st>>>(M, N, K, Act, W, trans,
+    launch_dep(k_gemm_split<BN, ST, TH, MINB>, grid, TH, smem, st, M, N, K, Act, W, trans,
                                                                N % 4 == 0 && epilogue_vectorizable(e), e, err);
     count_launch();
 }

@@ -28,6 +28,7 @@
 #include <mutex>
 
 #include "epilogue.cuh"
+#include "launch.cuh"
 #include "mp.cuh"
 #include "ptx.cuh"
 #include "tc.cuh"
@@ -62,6 +63,7 @@ __global__ void __launch_bounds__(256) k_gemm_tc(const __grid_constant__ CUtenso
                                                  const __grid_constant__ CUtensorMap tmB, int M, int N, int K,
                                                  int BN, int tmem_cols, int n_stages, int vec, int nseg, int kofs,
                                                  Epi e, int *err) {
+    dep_entry();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[TC_STAGES], bar_empty[TC_STAGES], bar_done;
     __shared__ uint32_t tmem_base_sh;
@@ -253,7 +255,7 @@ int launch_gemm_tc(int M, int N, int K, const __nv_bfloat16 *Act, const __nv_bfl
     cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     const int vec = epilogue_vectorizable(e);
     dim3 grid((M + TC_M - 1) / TC_M, N / BN);
-    k_gemm_tc<<<grid, 256, smem, st>>>(ma, mb, M, N, K, BN, tmem_cols, n_stages, vec, nseg, K, e, err);
+    launch_dep(k_gemm_tc, grid, 256, smem, st, ma, mb, M, N, K, BN, tmem_cols, n_stages, vec, nseg, K, e, err);
     count_launch();
     return 0;
 }

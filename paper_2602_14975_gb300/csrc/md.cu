@@ -4,6 +4,7 @@
 // and the piston kernels of the NPT path (Sec. 2, virial term in NPT). The
 // adjoint of the fast force with respect to its weights: distill.cu.
 #include <algorithm>
+#include "launch.cuh"
 #include "md.cuh"
 #include "mp.cuh"
 #include "ptx.cuh"
@@ -12,6 +13,7 @@ namespace dmts {
 
 // ---------------------------------------------------------- node helpers
 __global__ void k_embed(int n, int C, const uint8_t *species, const float *emb, float *s) {
+    dep_entry();
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (size_t)n * C) return;
     const int i = (int)(idx / C), c = (int)(idx % C);
@@ -21,12 +23,13 @@ __global__ void k_embed(int n, int C, const uint8_t *species, const float *emb, 
 void launch_embed(int n, int C, const uint8_t *species, const float *emb, float *s, cudaStream_t st) {
     if (n == 0) return;
     const size_t tot = (size_t)n * C;
-    k_embed<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n, C, species, emb, s);
+    launch_dep(k_embed, (unsigned)((tot + 255) / 256), 256, 0, st, n, C, species, emb, s);
     count_launch();
 }
 
 // e_atom[i] = scale * sum_c u[i][c]  (warp per atom)
 __global__ void k_rowsum(int n, int C, const float *u, float scale, float *e_atom) {
+    dep_entry();
     const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= n) return;
     float s = 0.f;
@@ -37,7 +40,7 @@ __global__ void k_rowsum(int n, int C, const float *u, float scale, float *e_ato
 
 void launch_rowsum(int n, int C, const float *u, float scale, float *e_atom, cudaStream_t st) {
     if (n == 0) return;
-    k_rowsum<<<(n + 7) / 8, 256, 0, st>>>(n, C, u, scale, e_atom);
+    launch_dep(k_rowsum, (n + 7) / 8, 256, 0, st, n, C, u, scale, e_atom);
     count_launch();
 }
 
@@ -205,6 +208,7 @@ struct NCHeadSmem {
 
 template <int K, int NC, int NL>
 __global__ void __launch_bounds__(NCH_WARPS * 32) k_nc_head(NCHeadArgs g) {
+    dep_entry(g.n_atoms <= (int)gridDim.x);
     using SM = NCHeadSmem<K, NC, NL>;
     constexpr int H = SM::H, QKW = SM::QKW, RSTR = SM::RSTR;
     extern __shared__ __align__(16) unsigned char nch_smem[];
@@ -557,7 +561,7 @@ static void nc_head_launch(const NCHeadArgs &a, cudaStream_t st) {
                                                     NCH_WARPS * 32, SM::bytes, dev));
     }
     const int blocks = std::min((a.n_atoms + NCH_WARPS - 1) / NCH_WARPS, resident);
-    k_nc_head<K, NC, NL><<<blocks, NCH_WARPS * 32, SM::bytes, st>>>(a);
+    launch_dep(k_nc_head<K, NC, NL>, blocks, NCH_WARPS * 32, SM::bytes, st, a);
     count_launch();
 }
 
@@ -755,6 +759,7 @@ void launch_mean_sub(const float *F_in, float *F_out, const int *rep_off, int n_
 // 64-bit atomics; integer sums do not depend on their order).
 __global__ void k_nc_convert(int n, const int *__restrict__ atom_rep, unsigned long long *__restrict__ Ffix,
                              float *__restrict__ F, unsigned long long *__restrict__ sum, unsigned *__restrict__ next) {
+    dep_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0 && next) *next = 0u;   // the head's work counter, for its next launch
     const bool live = i < n;
@@ -777,7 +782,7 @@ __global__ void k_nc_convert(int n, const int *__restrict__ atom_rep, unsigned l
 void launch_nc_convert(int n, const int *atom_rep, unsigned long long *Ffix, float *F, unsigned long long *sum,
                        unsigned *next, cudaStream_t st) {
     if (n == 0) return;
-    k_nc_convert<<<(n + 255) / 256, 256, 0, st>>>(n, atom_rep, Ffix, F, sum, next);
+    launch_dep(k_nc_convert, (n + 255) / 256, 256, 0, st, n, atom_rep, Ffix, F, sum, next);
     count_launch();
 }
 
@@ -786,6 +791,7 @@ __global__ void k_nc_apply(int n, const int *__restrict__ atom_rep, const int *_
                            const float *__restrict__ F, float *__restrict__ F_out,
                            const unsigned long long *__restrict__ sum, double *__restrict__ net,
                            const int *__restrict__ err) {
+    dep_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (net && i < 3 * n_rep) net[i] = fix_sum_to_double(sum[i]);
     if (i >= n || *err) return;
@@ -800,7 +806,7 @@ void launch_nc_apply(int n, const int *atom_rep, const int *rep_off, int n_rep, 
                      const unsigned long long *sum, double *net, const int *err, cudaStream_t st) {
     const int work = n > 3 * n_rep ? n : 3 * n_rep;
     if (work == 0) return;
-    k_nc_apply<<<(work + 255) / 256, 256, 0, st>>>(n, atom_rep, rep_off, n_rep, F, F_out, sum, net, err);
+    launch_dep(k_nc_apply, (work + 255) / 256, 256, 0, st, n, atom_rep, rep_off, n_rep, F, F_out, sum, net, err);
     count_launch();
 }
 
@@ -809,6 +815,7 @@ void launch_nc_apply(int n, const int *atom_rep, const int *rep_off, int n_rep, 
 // are not bonded; LJ between heavy atoms of different molecules,
 // 4 eps ((s/r)^12 - (s/r)^6) f(r/lj_rc; p); plus bonds.
 __global__ void __launch_bounds__(128) k_prior(PriorArgs g) {
+    dep_entry();
     __shared__ int sh_queue[4][64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wa = blockIdx.x * 4 + warp;
@@ -873,7 +880,7 @@ __global__ void __launch_bounds__(128) k_prior(PriorArgs g) {
 
 void launch_prior(const PriorArgs &a, cudaStream_t st) {
     if (a.n_atoms == 0) return;
-    k_prior<<<(a.n_atoms + 3) / 4, 128, 0, st>>>(a);
+    launch_dep(k_prior, (a.n_atoms + 3) / 4, 128, 0, st, a);
     count_launch();
 }
 
@@ -891,6 +898,7 @@ __device__ __forceinline__ void outer_kick(float h, float lx, float ly, float lz
 // One thread per atom; the operations selected by `ops` run in this order:
 // closing B, closing outer kick, opening outer kick, then B-A-O-A.
 __global__ void k_integrate(IntegArgs g) {
+    dep_entry();
     if (*g.err) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.n_atoms) return;
@@ -973,7 +981,7 @@ __global__ void k_integrate(IntegArgs g) {
 
 void launch_integrate(const IntegArgs &a, cudaStream_t st) {
     if (a.n_atoms == 0) return;
-    k_integrate<<<(a.n_atoms + 255) / 256, 256, 0, st>>>(a);
+    launch_dep(k_integrate, (a.n_atoms + 255) / 256, 256, 0, st, a);
     count_launch();
 }
 
@@ -1108,6 +1116,7 @@ void launch_baro_end(const BaroArgs &a, cudaStream_t st) {
 }
 
 __global__ void k_advance(uint64_t *step, int n_rep, uint64_t add, const int *err) {
+    dep_entry();
     if (*err) return;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r < n_rep) step[r] += add;
@@ -1115,7 +1124,7 @@ __global__ void k_advance(uint64_t *step, int n_rep, uint64_t add, const int *er
 
 void launch_advance_step(uint64_t *step, int n_rep, uint64_t add, const int *err, cudaStream_t st) {
     if (n_rep == 0) return;
-    k_advance<<<(n_rep + 127) / 128, 128, 0, st>>>(step, n_rep, add, err);
+    launch_dep(k_advance, (n_rep + 127) / 128, 128, 0, st, step, n_rep, add, err);
     count_launch();
 }
 

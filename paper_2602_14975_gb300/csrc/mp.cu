@@ -8,6 +8,7 @@
 
 #include "edge.cuh"
 #include "epilogue.cuh"
+#include "launch.cuh"
 #include "mp.cuh"
 #include "pack.cuh"
 #include "ptx.cuh"
@@ -15,6 +16,7 @@
 namespace dmts {
 
 constexpr int MP_WARPS = 4;
+constexpr unsigned kOneWave = 1024;   // warps that are all resident from the start (launch.cuh)
 
 // ------------------------------------------------------------------ forward
 // Warp per receiver i, lane owns CPW consecutive channels c = lane*CPW + u.
@@ -24,6 +26,7 @@ constexpr int MP_WARPS = 4;
 // owns CW = C / SPLIT channels, offset co = part * CW.
 template <int C, int LMAX, int K, int SPLIT>
 __global__ void __launch_bounds__(MP_WARPS * 32) k_mp_fwd(EdgeGeom g, LayerIO io) {
+    dep_entry(gridDim.x <= kOneWave / MP_WARPS);
     constexpr int NL = LMAX + 1, NLM = NL * NL, CW = C / SPLIT, CPW = CW / 32;
     using T = typename Pack<CPW>::T;
     constexpr int NP = Pack<CPW>::NP, PW = Pack<CPW>::W;
@@ -215,6 +218,7 @@ __device__ __forceinline__ void ld_rec(const float4 *p, T *v) {
 
 template <int C, int LMAX, int K, bool VIR>
 __global__ void __launch_bounds__(32) k_mp_bwd(EdgeGeom g, LayerIO io) {
+    dep_entry(gridDim.x <= kOneWave);
     using S = BwdSmem<C, LMAX, K>;
     using T = typename S::T;
     constexpr int NL = S::NL, NLM = S::NLM, CPW = S::CPW, NP = S::NP, PW = Pack<CPW>::W, V4 = S::V4, KY = S::KY;
@@ -506,6 +510,7 @@ __global__ void __launch_bounds__(32) k_mp_bwd(EdgeGeom g, LayerIO io) {
 // the words cleared for the next evaluation (also after an aborted one).
 __global__ void k_fix_convert(int n, unsigned long long *__restrict__ Ffix, float *__restrict__ F,
                               unsigned long long *__restrict__ Wfix, float *__restrict__ W) {
+    dep_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
 #pragma unroll
@@ -524,7 +529,7 @@ __global__ void k_fix_convert(int n, unsigned long long *__restrict__ Ffix, floa
 void launch_fix_convert(int n, unsigned long long *Ffix, float *F, unsigned long long *Wfix, float *W,
                         cudaStream_t st) {
     if (n == 0) return;
-    k_fix_convert<<<(n + 255) / 256, 256, 0, st>>>(n, Ffix, F, Wfix, W);
+    launch_dep(k_fix_convert, (n + 255) / 256, 256, 0, st, n, Ffix, F, Wfix, W);
     count_launch();
 }
 
@@ -534,7 +539,7 @@ template <int C, int LMAX>
 static void fwd_c(const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
     constexpr int SP = C >= 128 ? 2 : 1;
     const int blocks = (g.n_atoms + MP_WARPS - 1) / MP_WARPS;
-    k_mp_fwd<C, LMAX, 8, SP><<<dim3(blocks, SP), MP_WARPS * 32, 0, st>>>(g, io);
+    launch_dep_if(blocks <= (int)kOneWave / MP_WARPS, k_mp_fwd<C, LMAX, 8, SP>, dim3(blocks, SP), MP_WARPS * 32, 0, st, g, io);
     count_launch();
 }
 
@@ -542,7 +547,7 @@ template <int C, int LMAX, bool VIR>
 static void bwd_launch(const EdgeGeom &g, const LayerIO &io, cudaStream_t st) {
     constexpr size_t smem = sizeof(BwdSmem<C, LMAX, 8>);
     static_assert(smem <= 48 * 1024, "shared memory without an opt-in");
-    k_mp_bwd<C, LMAX, 8, VIR><<<g.n_atoms, 32, smem, st>>>(g, io);
+    launch_dep_if(g.n_atoms <= (int)kOneWave, k_mp_bwd<C, LMAX, 8, VIR>, g.n_atoms, 32, smem, st, g, io);
     count_launch();
 }
 
@@ -584,6 +589,7 @@ constexpr int GEMM_KC = 32, GEMM_LD = GEMM_KC + 4, GEMM_STAGES = 3;
 template <int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_f32(int M, int N, int K, const float *__restrict__ Act,
                                                                    const float *__restrict__ W, int trans, int vec, Epi e) {
+    dep_entry();
     constexpr int THREADS = (BM / TM) * (BN / TN), TY = BM / TM, TX = BN / TN, CH = GEMM_KC / 4;
     extern __shared__ __align__(16) float gemm_smem[];
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
@@ -694,7 +700,7 @@ static void gemm_f32_launch(int M, int N, int K, const float *Act, const float *
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_gemm_f32<BM, BN, TM, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
-    k_gemm_f32<BM, BN, TM, TN><<<grid, (BM / TM) * (BN / TN), smem, st>>>(M, N, K, Act, W, trans, N % 4 == 0 && epilogue_vectorizable(e), e);
+    launch_dep(k_gemm_f32<BM, BN, TM, TN>, grid, (BM / TM) * (BN / TN), smem, st, M, N, K, Act, W, trans, N % 4 == 0 && epilogue_vectorizable(e), e);
     count_launch();
 }
 
@@ -720,6 +726,7 @@ void launch_gemm_f32(int M, int N, int K, const float *Act, const float *W, int 
 // -------------------------------------------------- per-replica FP64 sums
 __global__ void k_replica_sum(const float *__restrict__ v, const int *__restrict__ rep_off,
                               double *__restrict__ out, int accumulate) {
+    dep_entry();
     __shared__ double red[32];
     const int r = blockIdx.x;
     const int beg = rep_off[r], end = rep_off[r + 1];
@@ -747,7 +754,7 @@ __global__ void k_replica_sum(const float *__restrict__ v, const int *__restrict
 void launch_replica_sum(const float *v, const int *rep_off, int n_rep, double *out, int accumulate,
                         cudaStream_t st) {
     if (n_rep == 0) return;
-    k_replica_sum<<<n_rep, 1024, 0, st>>>(v, rep_off, out, accumulate);
+    launch_dep(k_replica_sum, n_rep, 1024, 0, st, v, rep_off, out, accumulate);
     count_launch();
 }
 

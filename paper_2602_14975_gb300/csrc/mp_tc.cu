@@ -18,6 +18,7 @@
 #include <cuda_fp16.h>
 
 #include "edge.cuh"
+#include "launch.cuh"
 #include "mp.cuh"
 #include "ptx.cuh"
 #include "tc.cuh"
@@ -324,6 +325,7 @@ constexpr size_t fwd_tc_tiles() { return S_BYTES + TcDims<LMAX>::e_bytes + 1024;
 // tensor memory and returns.
 template <int LMAX>
 __global__ void __launch_bounds__(TC_THREADS, 3) k_mp_fwd_tc(EdgeGeom g, LayerIO io, float escale, int *err) {
+    dep_entry(g.n_atoms <= (int)gridDim.x);
     using D = TcDims<LMAX>;
     constexpr int NL = D::NL, NLM = D::NLM, C = TC_C;
     constexpr int TMEM = 128;   // columns allocated; NN <= 80 used
@@ -515,6 +517,7 @@ __global__ void __launch_bounds__(TC_THREADS, 3) k_mp_fwd_tc(EdgeGeom g, LayerIO
 // s 2^(TC_TOP - e).
 __global__ void __launch_bounds__(256) k_feature_split(int n, const float *__restrict__ s, __half *__restrict__ s16,
                                                        int *__restrict__ s_exp) {
+    dep_entry();
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= n) return;
     const float4 v = __ldg(reinterpret_cast<const float4 *>(s + (size_t)i * TC_C) + lane);
@@ -554,7 +557,7 @@ void fwd_tc_launch(const EdgeGeom &g, const LayerIO &io, int *err, cudaStream_t 
     cudaFuncSetAttribute(k_mp_fwd_tc<LMAX>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
     const int grid = std::min(g.n_atoms, persistent_grid(reinterpret_cast<const void *>(k_mp_fwd_tc<LMAX>), TC_THREADS, smem, 128));
-    k_mp_fwd_tc<LMAX><<<grid, TC_THREADS, smem, st>>>(g, io, basis_scale(g), err);
+    launch_dep_if(g.n_atoms <= grid, k_mp_fwd_tc<LMAX>, grid, TC_THREADS, smem, st, g, io, basis_scale(g), err);
     count_launch();
 }
 
@@ -582,7 +585,7 @@ bool mp_tc_supported(int C, int K) { return C == TC_C && K == TC_KR; }
 
 void launch_feature_split(int n, const float *s, void *s16, int *s_exp, cudaStream_t st) {
     if (n == 0) return;
-    k_feature_split<<<(n + 7) / 8, 256, 0, st>>>(n, s, static_cast<__half *>(s16), s_exp);
+    launch_dep(k_feature_split, (n + 7) / 8, 256, 0, st, n, s, static_cast<__half *>(s16), s_exp);
     count_launch();
 }
 

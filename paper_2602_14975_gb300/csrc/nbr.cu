@@ -4,6 +4,7 @@
 // index, so their order is canonical and independent of scheduling.
 #include <algorithm>
 
+#include "launch.cuh"
 #include "nbr.cuh"
 #include "ptx.cuh"
 
@@ -14,13 +15,14 @@ __device__ __forceinline__ bool gated_off(const int *gate, const int *err) {
 }
 
 __global__ void k_atom_rep(const int *rep_off, int n_rep, int n, int *atom_rep) {
+    dep_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) atom_rep[i] = replica_of(rep_off, n_rep, i);
 }
 
 void atom_rep_map(const int *rep_off, int n_rep, int n_atoms, int *atom_rep, cudaStream_t st) {
     if (n_atoms == 0) return;
-    k_atom_rep<<<(n_atoms + 255) / 256, 256, 0, st>>>(rep_off, n_rep, n_atoms, atom_rep);
+    launch_dep(k_atom_rep, (n_atoms + 255) / 256, 256, 0, st, rep_off, n_rep, n_atoms, atom_rep);
     count_launch();
 }
 
@@ -72,6 +74,7 @@ __device__ __forceinline__ void grid_open(const NbrWork &w, float r_list, int r)
     }
 }
 __global__ void k_grid_open(NbrWork w, float r_list) {
+    dep_entry();
     if (!gated_off(w.gate, w.err)) grid_open(w, r_list, blockIdx.x);
 }
 
@@ -95,6 +98,7 @@ __device__ __forceinline__ void cell_assign(const NbrWork &w, int i) {
     w.atom_slot[i] = atomicAdd(&w.cell_cnt[cell], 1);
 }
 __global__ void k_cell_assign(NbrWork w) {
+    dep_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < w.n_atoms && !gated_off(w.gate, w.err)) cell_assign(w, i);
 }
@@ -103,6 +107,7 @@ __device__ __forceinline__ void cell_scatter(const NbrWork &w, int i) {
     w.cell_atoms[w.cell_start[w.atom_cell[i]] + w.atom_slot[i]] = i;
 }
 __global__ void k_cell_scatter(NbrWork w) {
+    dep_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < w.n_atoms && !gated_off(w.gate, w.err)) cell_scatter(w, i);
 }
@@ -462,6 +467,7 @@ __device__ __forceinline__ void count_cell(const NbrWork &w, float rc2, float rc
     }
 }
 __global__ void __launch_bounds__(NBC_WARPS * 32) k_nbr_count_cell(NbrWork w, float rc2, float rc2_sub) {
+    dep_entry();
     __shared__ CountSmem sm;
     if (!gated_off(w.gate, w.err)) count_cell(w, rc2, rc2_sub, blockIdx.x, sm);
 }
@@ -549,6 +555,7 @@ __device__ __forceinline__ void fill_row(const NbrWork &w, float rc2, const int 
 __global__ void __launch_bounds__(NB_WARPS * 32) k_nbr_fill_warp(NbrWork w, float rc2, const int *row_ptr, int *col,
                                                                  float *x_ref, float rc2_sub, const int *sub_row,
                                                                  int *sub_col) {
+    dep_entry();
     if (gated_off(w.gate, w.err)) return;
     __shared__ __align__(16) int buf[NB_WARPS][NB_MAXROW];
     const int warp = threadIdx.x >> 5, i = blockIdx.x * NB_WARPS + warp;
@@ -669,6 +676,7 @@ __device__ __forceinline__ void scan_tile(const ScanJob &J, int n, int n_tiles, 
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan(ScanJob j0, ScanJob j1, int n, int n_tiles,
                                                        unsigned long long *status_all, unsigned long long *counters,
                                                        int tiles_cap, int *err, const int *gate) {
+    dep_entry();
     if (gated_off(gate, err)) return;
     scan_tile(blockIdx.y ? j1 : j0, n, n_tiles, status_all + (size_t)blockIdx.y * tiles_cap, counters + blockIdx.y, err);
 }
@@ -678,20 +686,20 @@ void scan_ints(const NbrWork &w, const int *in0, int *out0, long long cap0, long
     const int tiles = (n + kScanTile - 1) / kScanTile;
     const int n_tiles = tiles > 0 ? tiles : 1;
     dim3 grid(n_tiles, in1 ? 2 : 1);
-    k_scan<<<grid, SCAN_THREADS, 0, st>>>(ScanJob{in0, out0, cap0, total0}, ScanJob{in1, out1, cap1, total1}, n,
+    launch_dep(k_scan, grid, SCAN_THREADS, 0, st, ScanJob{in0, out0, cap0, total0}, ScanJob{in1, out1, cap1, total1}, n,
                                           n_tiles, w.scan_status, w.scan_counter, w.scan_tiles, w.err, w.gate);
     count_launch();
 }
 
 void nbr_cells(const NbrWork &w, float r_list, cudaStream_t st) {
     if (w.n_atoms == 0) return;
-    k_grid_open<<<w.n_rep, 256, 0, st>>>(w, r_list);
+    launch_dep(k_grid_open, w.n_rep, 256, 0, st, w, r_list);
     count_launch();
     const int nb = (w.n_atoms + 255) / 256;
-    k_cell_assign<<<nb, 256, 0, st>>>(w);
+    launch_dep(k_cell_assign, nb, 256, 0, st, w);
     count_launch();
     scan_ints(w, w.cell_cnt, w.cell_start, -1, nullptr, nullptr, nullptr, -1, nullptr, w.n_cells, st);
-    k_cell_scatter<<<nb, 256, 0, st>>>(w);
+    launch_dep(k_cell_scatter, nb, 256, 0, st, w);
     count_launch();
 }
 
@@ -701,13 +709,13 @@ void nbr_fill(const NbrWork &w, float r_list, int *row_ptr, int *col, long long 
     const int nb = (w.n_atoms + NB_WARPS - 1) / NB_WARPS;
     NbrWork wc = w;
     if (!sub_row) wc.counts_sub = nullptr;
-    k_nbr_count_cell<<<wc.n_cells, NBC_WARPS * 32, 0, st>>>(wc, r_list * r_list, r_sub * r_sub);
+    launch_dep(k_nbr_count_cell, wc.n_cells, NBC_WARPS * 32, 0, st, wc, r_list * r_list, r_sub * r_sub);
     count_launch();
     // the full list's and the sub-list's row offsets in one launch
     scan_ints(wc, wc.counts, row_ptr, capacity, wc.total, wc.counts_sub, wc.counts_sub ? sub_row : nullptr,
               sub_capacity, nullptr, wc.n_atoms, st);
     if (col) {
-        k_nbr_fill_warp<<<nb, NB_WARPS * 32, 0, st>>>(wc, r_list * r_list, row_ptr, col, x_ref, r_sub * r_sub,
+        launch_dep(k_nbr_fill_warp, nb, NB_WARPS * 32, 0, st, wc, r_list * r_list, row_ptr, col, x_ref, r_sub * r_sub,
                                                       wc.counts_sub ? sub_row : nullptr,
                                                       wc.counts_sub ? sub_col : nullptr);
         count_launch();
