@@ -731,8 +731,10 @@ void nbr_fill(const NbrWork &w, float r_list, int *row_ptr, int *col, long long 
 // Barrier: block b > 0 writes the epoch (launch number, phase) to its word and
 // waits for block 0's release word; block 0 collects the words, reads the
 // error word once for everybody and releases with a stop bit. Every wait is
-// bounded; words of an earlier launch never match.
+// bounded, by more than a long kernel of another stream can keep the last
+// blocks from starting; words of an earlier launch never match.
 constexpr int RB_THREADS = NBC_WARPS * 32;
+constexpr uint64_t RB_WAIT_NS = 10 * kWaitLimitNs;
 static_assert(RB_THREADS == SCAN_THREADS, "one block shape for every phase");
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
@@ -754,7 +756,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned epoch, int
         for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
             const uint64_t t0 = globaltimer_ns();
             while (b > 0 && ok && ld_acquire(words + b) != epoch)
-                if (globaltimer_ns() - t0 > kWaitLimitNs) ok = 0;
+                if (globaltimer_ns() - t0 > RB_WAIT_NS) ok = 0;
         }
         ok = __syncthreads_and(ok);
         if (threadIdx.x == 0) {
@@ -770,7 +772,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned epoch, int
         unsigned v;
         bool ok = true;
         while (((v = ld_acquire(release)) >> 1) != epoch && ok)
-            if (globaltimer_ns() - t0 > 2 * kWaitLimitNs) ok = false;
+            if (globaltimer_ns() - t0 > 2 * RB_WAIT_NS) ok = false;
         if (!ok) set_error(err, DMTS_E_TIMEOUT);
         go = ok && !(v & 1u);
         __threadfence();
