@@ -41,14 +41,15 @@ PROF_EVERY = 4   # time every 4th outer step of the timed region per kernel
 KCAL_A3_PER_ATM = 101325.0 * 6.02214076e23 * 1e-30 / 4184.0   # 1 atm in kcal/mol/A^3
 
 NCU_TRAFFIC = {
-    "mp_bwd": {"bytes_per_launch": (154229760 + 19248896 + 154260992 + 16390400 + 139650304 + 268544) / 3,
-               # the adjoint's code: channel-pack helpers, kernel, the argument
-               # structs, the device helpers
+    "mp_bwd": {"bytes_per_launch": (154136576 + 19699968 + 154156800 + 16406272) / 2,
+               # the adjoint's code: channel-pack and geometry helpers, kernel, the
+               # argument structs, the device helpers
                "sources": [("paper_2602_14975_gb300/csrc/pack.cuh", None),
+                           ("paper_2602_14975_gb300/csrc/edge.cuh", None),
                            ("paper_2602_14975_gb300/csrc/mp.cu", ("// ---- adjoint", "// In the forward pass")),
                            ("paper_2602_14975_gb300/csrc/mp.cuh", ("struct EdgeGeom {", "template <int CPW>")),
                            ("paper_2602_14975_gb300/csrc/common.cuh", None)],
-               "sha256": "8c1a3a7c5d60e748369169f7e9198032650ff7e2427e60f09026a2b70bc7c32c"},
+               "sha256": "48145d82330d8d686458510e2e0db0e2db9e66cac1ece6e52e59a4de45c2ee3f"},
 }
 
 
