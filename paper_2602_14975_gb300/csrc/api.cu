@@ -341,7 +341,6 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
     __nv_bfloat16 *s_bf = bf ? (__nv_bfloat16 *)w.s_bf.p : nullptr, *gz_bf = bf ? (__nv_bfloat16 *)w.gz_bf.p : nullptr;
     __nv_bfloat16 *gs0_bf = bf ? (__nv_bfloat16 *)w.gs0_bf.p : nullptr, *gs1_bf = bf ? (__nv_bfloat16 *)w.gs1_bf.p : nullptr;
     const EdgeGeom g = edge_geom(s, row_ptr, col, m);
-    if (!(flags & kFlagEmbedded)) { ProfScope ps(ctx, "embed", st); launch_embed(N, C, s.species, m.emb, S, st); }
     for (int t = 0; t < L; ++t) {
         LayerIO io;
         memset(&io, 0, sizeof io);
@@ -380,7 +379,8 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
             return DMTS_E_CUDA;
         Epi e2 = epi(EPI_RESID);
         e2.bias = m.b2[t];
-        e2.res = S + nc_ * t;
+        e2.res = t == 0 ? m.emb : S + nc_ * t;   // s^0 is the species embedding
+        e2.res_row = t == 0 ? s.species : nullptr;
         e2.out = S + nc_ * (t + 1);
         e2.out_bf16 = t == L - 1 ? s_bf : nullptr;
         if (!contract(ctx, m, N, C, C, act, act_bf, m.w2[t], 1, m.w2_bf[t], e2, st, "gemm_tc", "gemm"))
@@ -496,7 +496,7 @@ dmts_status nc_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const i
     Workspace &w = ctx->ws;
     const size_t nc_ = (size_t)N * C;
     const bool bf = m.bf16;
-    if (!w.nc_s.ensure(sizeof(float) * nc_ * 2) ||
+    if (!w.nc_s.ensure(sizeof(float) * nc_) ||
         !w.nc_q.ensure(sizeof(float) * nc_ * 2) ||
         !w.nc_act.ensure(sizeof(float) * nc_) || !w.nc_qk.ensure(sizeof(float) * (size_t)N * QKW) ||
         !w.nc_v.ensure(sizeof(float) * (size_t)N * nc_v_stride(m.nl)) || !w.nc_f.ensure(sizeof(float) * 3 * (N + 1)) ||
@@ -511,9 +511,8 @@ dmts_status nc_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const i
     __nv_bfloat16 *q_bf = bf ? (__nv_bfloat16 *)w.nc_q_bf.p : nullptr;
     __nv_bfloat16 *act_bf = bf ? (__nv_bfloat16 *)w.nc_act_bf.p : nullptr;
     __nv_bfloat16 *s_bf = bf ? (__nv_bfloat16 *)w.nc_s_bf.p : nullptr;
-    float *s0 = (float *)w.nc_s.p, *s1 = s0 + nc_;
+    float *s1 = (float *)w.nc_s.p;
     const EdgeGeom g = edge_geom(s, row_ptr, col, m);
-    if (!(flags & kFlagEmbedded)) { ProfScope ps(ctx, "embed", st); launch_embed(N, C, s.species, m.emb, s0, st); }
     FirstIO io = first_io(ctx, s, m);
     io.A = (flags & kFlagKeepPre) ? (float *)w.dist_A.p : nullptr;   // the head needs q and V only; kept for the distillation
     io.T = (flags & kFlagKeepPre) ? (float *)w.dist_T.p : nullptr;
@@ -536,7 +535,8 @@ dmts_status nc_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const i
         return DMTS_E_CUDA;
     Epi e2 = epi(EPI_RESID);
     e2.bias = m.b2[0];
-    e2.res = s0;
+    e2.res = m.emb;   // s^0 is the species embedding
+    e2.res_row = s.species;
     e2.out = s1;
     e2.out_bf16 = s_bf;
     if (!contract(ctx, m, N, C, C, (float *)w.nc_act.p, act_bf, m.w2[0], 1, m.w2_bf[0], e2, st, "nc_gemm_tc", "nc_gemm"))
@@ -1043,7 +1043,7 @@ dmts_status energy_forces_cons(dmts_ctx *ctx, const dmts_system *sys, const dmts
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     SysView v = make_view(ctx, sys, st);
-    s = cons_eval(ctx, v, nbr->row_ptr, nbr->col, energy, forces, flags & ~kFlagEmbedded, st, virial);
+    s = cons_eval(ctx, v, nbr->row_ptr, nbr->col, energy, forces, flags, st, virial);
     if (s != DMTS_OK) return s;
     return ck(ctx, cudaGetLastError(), "energy_forces_cons launch") ? DMTS_OK : DMTS_E_CUDA;
 }
@@ -1060,7 +1060,7 @@ dmts_status forces_nc(dmts_ctx *ctx, const dmts_system *sys, const dmts_nbr *nbr
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     SysView v = make_view(ctx, sys, st);
-    s = nc_eval(ctx, v, nbr->row_ptr, nbr->col, forces, net_force, flags & ~kFlagEmbedded, st, virial, 0);
+    s = nc_eval(ctx, v, nbr->row_ptr, nbr->col, forces, net_force, flags, st, virial, 0);
     if (s != DMTS_OK) return s;
     return ck(ctx, cudaGetLastError(), "forces_nc launch") ? DMTS_OK : DMTS_E_CUDA;
 }
@@ -1137,7 +1137,7 @@ dmts_status nc_distill_step(dmts_ctx *ctx, const dmts_system *sys, const dmts_nb
     float *dw = grad ? grad : (float *)w.dist_dw.p;
     if (!ck(ctx, cudaMemsetAsync(dw, 0, sizeof(float) * nb, st), "gradient reset")) return DMTS_E_CUDA;
     auto at = [&](const float *p) { return dw + (p - m.dev); };
-    const float *s1 = (const float *)w.nc_s.p + (size_t)N * C;
+    const float *s1 = (const float *)w.nc_s.p;
     float *part_buf = (float *)w.dist_part.p;
     if (fit_qk) launch_atb(N, QKW, C, gqk, s1, at(m.Wqk), nullptr, part_buf, st);   // dW_qk = gQK^T s1
     // Gradients are sums over the batch: here the split contractions go by the
@@ -1347,13 +1347,9 @@ dmts_status dmts::respa_run(dmts_ctx *ctx, dmts_state *stt, const dmts_integrato
     const SysView v = state_view(stt);
     const int *crow = (int *)si->cons_row.p, *ccol = (int *)si->cons_col.p;
     const int *nrow = (int *)si->nc_row.p, *ncol = (int *)si->nc_col.p;
-    // the species embedding is computed by the first evaluation of each
-    // model in this call and kept in the workspace for the others
-    int cons_emb = 0, nc_emb = 0;
     auto cons_full = [&]() {
-        const dmts_status r = cons_eval(ctx, v, crow, ccol, stt->energy, stt->f_cons, DMTS_WITH_PRIOR | cons_emb, st,
+        const dmts_status r = cons_eval(ctx, v, crow, ccol, stt->energy, stt->f_cons, DMTS_WITH_PRIOR, st,
                                         stt->virial_cons);
-        cons_emb = kFlagEmbedded;
         return r;
     };
     // fast force; inside the inner loop it also adds its virial proxy to the
@@ -1364,9 +1360,8 @@ dmts_status dmts::respa_run(dmts_ctx *ctx, dmts_state *stt, const dmts_integrato
     // stt->f_nc: one launch and one pass over the forces less per inner step.
     bool mean_pending = false;
     auto nc_fast_on = [&](bool with_virial, cudaStream_t s_nc) {
-        const dmts_status r = nc_eval(ctx, v, nrow, ncol, stt->f_nc, nullptr, DMTS_WITH_BONDS | nc_emb | kFlagDeferMean,
+        const dmts_status r = nc_eval(ctx, v, nrow, ncol, stt->f_nc, nullptr, DMTS_WITH_BONDS | kFlagDeferMean,
                                       s_nc, with_virial ? stt->virial_nc : nullptr, 1);
-        nc_emb = kFlagEmbedded;
         mean_pending = true;
         return r;
     };
@@ -1685,10 +1680,6 @@ dmts_status dmts::respa_run(dmts_ctx *ctx, dmts_state *stt, const dmts_integrato
         return DMTS_E_CUDA;
     const cudaStream_t user_st = st;
     st = ctx->gstream;
-    // the workspace's species embedding may be another state's by the time
-    // the graph is replayed: the captured call computes its own
-    cons_emb = 0;
-    nc_emb = 0;
     const unsigned long long l0 = launch_count();
     if (!ck(ctx, cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed), "graph capture")) {
         st = user_st;

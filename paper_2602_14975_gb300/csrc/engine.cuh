@@ -192,11 +192,6 @@ struct dmts_ctx {
 namespace dmts {
 bool ck(dmts_ctx *ctx, cudaError_t e, const char *what);
 dmts_status fail(dmts_ctx *ctx, dmts_status s, const std::string &msg);
-// Internal flag of cons_eval / nc_eval: the layer-0 features (the species
-// embedding) already in the workspace belong to this system, so the
-// embedding is not recomputed (set within one respa_step call, where the
-// species do not change).
-constexpr int kFlagEmbedded = 1 << 30;
 // Internal flag of nc_eval: keep the layer output A (ws.dist_A) and the MLP
 // pre-activation (ws.dist_h) for the distillation's backward pass.
 constexpr int kFlagKeepPre = 1 << 29;

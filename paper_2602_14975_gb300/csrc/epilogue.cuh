@@ -11,6 +11,13 @@ namespace dmts {
 // store, so that many loads are in flight per warp.
 constexpr int EU = 4;
 
+// Row of the residual input. The first layer's is the species embedding, read
+// from the table itself: an [M][N] copy of it was a launch of its own (12 us at
+// 49,152 rows of 64, 3 us at 80) and M N floats written and read.
+__device__ __forceinline__ size_t res_offset(const Epi &e, int m, int N) {
+    return (size_t)(e.res_row ? (int)__ldg(e.res_row + m) : m) * N;
+}
+
 __device__ __forceinline__ void epilogue_tile(const Epi &e, int N, int rows, int m0, int n0, int BN,
                                               const float *tile, int ld) {
     const int total = rows * BN;
@@ -58,7 +65,7 @@ __device__ __forceinline__ void epilogue_tile(const Epi &e, int N, int rows, int
             float rs[EU], b[EU];
 #pragma unroll
             for (int u = 0; u < EU; ++u) {
-                rs[u] = ok[u] ? __ldg(e.res + o[u]) : 0.f;
+                rs[u] = ok[u] ? __ldg(e.res + res_offset(e, m0 + r_[u], N) + n[u]) : 0.f;
                 b[u] = ok[u] ? __ldg(e.bias + n[u]) : 0.f;
             }
 #pragma unroll
@@ -205,7 +212,7 @@ __device__ __forceinline__ void epilogue_tile_v4(const Epi &e, int N, int rows, 
             float4 rs[EU4];
 #pragma unroll
             for (int u = 0; u < EU4; ++u)
-                rs[u] = ok[u] ? ld4(e.res + (size_t)(m0 + rr[u]) * N + n0 + 4 * cc[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                rs[u] = ok[u] ? ld4(e.res + res_offset(e, m0 + rr[u], N) + n0 + 4 * cc[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int u = 0; u < EU4; ++u)
                 if (ok[u]) {

@@ -12,21 +12,6 @@
 namespace dmts {
 
 // ---------------------------------------------------------- node helpers
-__global__ void k_embed(int n, int C, const uint8_t *species, const float *emb, float *s) {
-    dep_entry();
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)n * C) return;
-    const int i = (int)(idx / C), c = (int)(idx % C);
-    s[idx] = emb[species[i] * C + c];
-}
-
-void launch_embed(int n, int C, const uint8_t *species, const float *emb, float *s, cudaStream_t st) {
-    if (n == 0) return;
-    const size_t tot = (size_t)n * C;
-    launch_dep(k_embed, (unsigned)((tot + 255) / 256), 256, 0, st, n, C, species, emb, s);
-    count_launch();
-}
-
 // e_atom[i] = scale * sum_c u[i][c]  (warp per atom)
 __global__ void k_rowsum(int n, int C, const float *u, float scale, float *e_atom) {
     dep_entry();

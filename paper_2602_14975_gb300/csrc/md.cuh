@@ -210,7 +210,6 @@ void launch_baro_start(const BaroArgs &a, cudaStream_t st);
 // end of an outer step: G from K and the estimator, half kick
 void launch_baro_end(const BaroArgs &a, cudaStream_t st);
 void launch_advance_step(uint64_t *step, int n_rep, uint64_t add, const int *err, cudaStream_t st);
-void launch_embed(int n, int C, const uint8_t *species, const float *emb, float *s, cudaStream_t st);
 void launch_rowsum(int n, int C, const float *u, float scale, float *e_atom, cudaStream_t st);
 
 }  // namespace dmts

@@ -141,7 +141,8 @@ struct Epi {
     __nv_bfloat16 *out_bf16;   // optional split-bf16 copy of out, [M][2N] (hi | lo)
     float *out2;
     const float *bias;
-    const float *res;          // residual input [M][N]
+    const float *res;          // residual input [M][N], or
+    const uint8_t *res_row;    // (when set) row res_row[m] of it for row m: the species embedding
     float *H;                  // pre-activation store (nullable) / load
     const float *A;            // EPI_GA
     const float *wo;           // EPI_READOUT
