@@ -164,7 +164,12 @@ static dmts_status load_model(dmts_ctx *ctx, const dmts_model *in, bool is_nc, D
         m.U = take((size_t)m.nl * C);
         m.Wqk = take((size_t)2 * H * m.nc * C);   // Wq rows then Wk rows: one [2 H n_c][C] matrix
         m.UW = take((size_t)m.nl * S * K);
+        // complete before the context is handed out: a non-blocking stream
+        // (the serving loop's, a caller's) does not wait for the legacy one
         launch_tensor_head_weights(C, S, m.nl, m.emb, m.wrad[0], m.U, m.UW, nullptr);
+        if (!ck(ctx, cudaGetLastError(), "tensor-head weights") ||
+            !ck(ctx, cudaStreamSynchronize(nullptr), "tensor-head weights"))
+            return DMTS_E_CUDA;
     }
     if (m.bf16) {
         // split-bf16 host copies, K-major: each output row of the logical
