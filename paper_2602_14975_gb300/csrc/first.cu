@@ -41,7 +41,7 @@ constexpr int FL_UNIT = 3;      // candidates per lane and sweep step, loaded to
 constexpr int FL_QUEUE = 128;   // at most 31 + 96 wait
 
 // Sweeps the row [beg, end): batch(n) is called with n <= 32 queued edges,
-// the e-th at queue[(taken + e) % 64] (displacement; w: 8 j + species).
+// the e-th at queue[(taken + e) % FL_QUEUE] (displacement; w: 8 j + species).
 template <class Fn>
 __device__ __forceinline__ void sweep_row(const EdgeGeom &g, const uint8_t *species, int n_species,
                                           const AtomGeom &a, int beg, int end, float4 *queue, int lane, Fn batch) {
@@ -94,7 +94,7 @@ struct FirstFwdSmem {
     static constexpr int TS = 2 * NLM * FL_K;
     // floats: weights, embedding, tensor-head weights; per warp: queue, records, T
     static constexpr int w_f = NL * FL_K * C;
-    static size_t bytes(int S) {
+    static constexpr size_t bytes(int S) {
         const size_t cta = w_f + (size_t)S * C + 4 * (size_t)S * FL_K;   // weights, embedding, tensor-head weights
         return 4 * (cta + WARPS * (4 * FL_QUEUE + 32 * RS + (size_t)S * TS + 4));
     }
@@ -276,7 +276,7 @@ struct FirstBwdSmem {
     static constexpr int NL = LMAX + 1, NLM = NL * NL, WARPS = 8;
     static constexpr int WS = C + 4;                            // weight row stride: eight rows in distinct banks
     static constexpr int QS = NLM * FL_K + 4;                   // Q of one species (rows of two species never collide)
-    static size_t bytes(int S) {
+    static constexpr size_t bytes(int S) {
         return 4 * ((size_t)NL * FL_K * WS + (size_t)S * C + WARPS * (4 * FL_QUEUE + NLM * C + (size_t)S * QS));
     }
 };
@@ -460,10 +460,17 @@ __global__ void k_tensor_head_weights(int C, int S, const float *emb, const floa
     if (lane == 0) UW[(h * S + z) * FL_K + k] = t;
 }
 
-// Persistent: as many CTAs as fit on the current device at once.
-template <class Kern>
-void first_launch(Kern kern, int warps, size_t smem, const EdgeGeom &g, const FirstIO &io, cudaStream_t st) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// Persistent: as many CTAs as fit on the current device at once. Shared memory
+// goes by the model's species, but the kernel's limit is the same whatever the
+// model: it is shared by all contexts, and a smaller model's host thread must
+// not lower it between another's setting and its launch.
+template <class SM, class Kern>
+void first_launch(Kern kern, const EdgeGeom &g, const FirstIO &io, cudaStream_t st) {
+    constexpr int warps = SM::WARPS;
+    constexpr size_t smem_max = SM::bytes(DMTS_MAX_SPECIES);
+    static_assert(smem_max <= 227 * 1024, "shared memory of the largest model");
+    const size_t smem = SM::bytes(io.n_species);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
     int dev = 0, n_sm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
@@ -475,14 +482,13 @@ void first_launch(Kern kern, int warps, size_t smem, const EdgeGeom &g, const Fi
 
 template <int C, int LMAX>
 void first_fwd_c(const EdgeGeom &g, const FirstIO &io, cudaStream_t st) {
-    first_launch(k_first_fwd<C, LMAX>, FirstFwdSmem<C, LMAX>::WARPS, FirstFwdSmem<C, LMAX>::bytes(io.n_species), g, io, st);
+    first_launch<FirstFwdSmem<C, LMAX>>(k_first_fwd<C, LMAX>, g, io, st);
 }
 
 template <int C, int LMAX>
 void first_bwd_c(const EdgeGeom &g, const FirstIO &io, cudaStream_t st) {
-    const size_t smem = FirstBwdSmem<C, LMAX>::bytes(io.n_species);
-    if (io.Wfix) first_launch(k_first_bwd<C, LMAX, true>, FirstBwdSmem<C, LMAX>::WARPS, smem, g, io, st);
-    else first_launch(k_first_bwd<C, LMAX, false>, FirstBwdSmem<C, LMAX>::WARPS, smem, g, io, st);
+    if (io.Wfix) first_launch<FirstBwdSmem<C, LMAX>>(k_first_bwd<C, LMAX, true>, g, io, st);
+    else first_launch<FirstBwdSmem<C, LMAX>>(k_first_bwd<C, LMAX, false>, g, io, st);
 }
 
 }  // namespace
