@@ -471,10 +471,7 @@ void first_launch(Kern kern, const EdgeGeom &g, const FirstIO &io, cudaStream_t 
     static_assert(smem_max <= 227 * 1024, "shared memory of the largest model");
     const size_t smem = SM::bytes(io.n_species);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-    int dev = 0, n_sm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const int fit = n_sm * resident_ctas(reinterpret_cast<const void *>(kern), warps * 32, smem, dev);
+    const int fit = sm_count() * resident_ctas(reinterpret_cast<const void *>(kern), warps * 32, smem, current_device());
     const int grid = std::min((g.n_atoms + warps - 1) / warps, fit);
     launch_dep(kern, grid, warps * 32, smem, st, g, io);
     count_launch();

@@ -247,13 +247,7 @@ static void gemm_split_launch(int M, int N, int K, const float *Act, const float
 void launch_gemm_split(int M, int N, int K, const float *Act, const float *W, int trans, const Epi &e, int *err,
                        cudaStream_t st) {
     if (M == 0) return;
-    static int n_sm = 0;
-    if (!n_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        n_sm = std::max(n_sm, 1);
-    }
+    const int n_sm = sm_count();
     // narrow tiles, 512 threads and two buffers while they fit on the GPU at
     // once: a force call of 80 atoms 252 us against 297, of 3,000 487 against
     // 534; the products and their order are the same

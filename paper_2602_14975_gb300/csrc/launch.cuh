@@ -22,15 +22,34 @@
 //  - while a graph is captured: its replays were slower with such edges (an
 //    outer step of 192 atoms 226 us against 214).
 #pragma once
+#include <algorithm>
 #include <utility>
 
 #include "common.cuh"
+#include "per_device.h"
 
 namespace dmts {
 
 __device__ __forceinline__ void dep_entry(bool early = true) {
     if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+inline int current_device() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return dev;
+}
+
+// SMs of the current device.
+inline int sm_count() {
+    static PerDevice sms;
+    const int dev = current_device();
+    return sms.get(dev, [dev] {
+        int n = 1;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return std::max(n, 1);
+    });
 }
 
 template <typename... P, typename... A>

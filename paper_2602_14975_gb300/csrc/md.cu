@@ -537,15 +537,13 @@ static void nc_head_launch(const NCHeadArgs &a, cudaStream_t st) {
     cudaFuncSetAttribute(k_nc_head<K, NC, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
     // persistent: as many warps as fit on the GPU at once, each taking every
     // (grid)-th atom
-    static int resident = 0;
-    if (!resident) {
-        int dev = 0, n_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        resident = std::max(1, n_sm * resident_ctas(reinterpret_cast<const void *>(k_nc_head<K, NC, NL>),
-                                                    NCH_WARPS * 32, SM::bytes, dev));
-    }
-    const int blocks = std::min((a.n_atoms + NCH_WARPS - 1) / NCH_WARPS, resident);
+    static PerDevice resident;
+    const int dev = current_device();
+    const int fit = resident.get(dev, [dev] {
+        return sm_count() * resident_ctas(reinterpret_cast<const void *>(k_nc_head<K, NC, NL>), NCH_WARPS * 32,
+                                          SM::bytes, dev);
+    });
+    const int blocks = std::min((a.n_atoms + NCH_WARPS - 1) / NCH_WARPS, fit);
     launch_dep(k_nc_head<K, NC, NL>, blocks, NCH_WARPS * 32, SM::bytes, st, a);
     count_launch();
 }

@@ -709,13 +709,7 @@ static void gemm_f32_launch(int M, int N, int K, const float *Act, const float *
 void launch_gemm_f32(int M, int N, int K, const float *Act, const float *W, int trans, const Epi &e,
                      cudaStream_t st) {
     if (M == 0) return;
-    static int n_sm = 0;
-    if (!n_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        n_sm = std::max(n_sm, 1);
-    }
+    const int n_sm = sm_count();
     // small tiles until the large ones give every SM two CTAs: at 4,000 rows
     // (N = K = 128) 10.4 us against 8.3 (plain) and 12.3 against 12.4 (SiLU
     // epilogue), at 192 rows 6.2 against 8.3, at 23,558 rows 41 against 27

@@ -544,10 +544,7 @@ float basis_scale(const EdgeGeom &g) {
 // CTAs to launch: as many as fit on the current device at once, and TMEM's
 // 512 columns per SM.
 int persistent_grid(const void *fn, int threads, size_t smem, int tmem_cols) {
-    int dev = 0, n_sm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    return n_sm * std::max(1, std::min(resident_ctas(fn, threads, smem, dev), 512 / tmem_cols));
+    return sm_count() * std::max(1, std::min(resident_ctas(fn, threads, smem, current_device()), 512 / tmem_cols));
 }
 
 template <int LMAX>

@@ -847,14 +847,13 @@ __global__ void __launch_bounds__(RB_THREADS) k_nbr_rebuild(NbrWork w, RebuildAr
 void nbr_rebuild(const NbrWork &w, float r_list, int *row_ptr, int *col, long long capacity, float *x_ref,
                  unsigned *sync, int *gate, cudaStream_t st, float r_sub, int *sub_row, int *sub_col,
                  long long sub_capacity) {
-    static int fit = 0;
-    if (!fit) {
-        int dev = 0, n_sm = 1, per_sm = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    // (found per device: a cooperative grid too large for the current one is refused)
+    static PerDevice resident;
+    const int fit = resident.get(current_device(), [] {
+        int per_sm = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nbr_rebuild, RB_THREADS, 0);
-        fit = std::max(1, std::min(n_sm * per_sm, kRebuildBlocks));
-    }
+        return std::max(1, std::min(sm_count() * per_sm, kRebuildBlocks));
+    });
     NbrWork wc = w;
     wc.gate = nullptr;
     if (!sub_row) wc.counts_sub = nullptr;
