@@ -159,7 +159,9 @@ __global__ void __launch_bounds__(TH, MINB) k_gemm_split(int M, int N, int K, co
         }
         tc_fence_before();
     };
-    auto wait = [&](int c) { return mbar_wait(bar + (ST == 2 ? 8 * (c & 1) : 0), ST == 2 ? (c >> 1) & 1 : c & 1) ? 1 : 0; };
+    auto bar_of = [&](int c) { return bar + (ST == 2 ? 8 * (c & 1) : 0); };
+    auto parity_of = [](int c) { return (uint32_t)(ST == 2 ? (c >> 1) & 1 : c & 1); };
+    auto wait = [&](int c) { return warp_wait(bar_of(c), parity_of(c)) ? 1 : 0; };   // (drain() loads TMEM warp-wide)
     int ok = 1, issued = 0;
     for (int c = 0; c < nk; ++c) {
         if (ST == 1 && c > 0) ok &= wait(c - 1);   // the tiles' last readers are done
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(TH, MINB) k_gemm_split(int M, int N, int K, co
         if (tid == 0) {
             set_error(err, (int)DMTS_E_TIMEOUT);
             // the MMAs issued, once more
-            for (int c = max(0, issued - ST); c < issued; ++c) wait(c);
+            for (int c = max(0, issued - ST); c < issued; ++c) mbar_wait(bar_of(c), parity_of(c));
         }
     } else {
         drain(nk - 1);

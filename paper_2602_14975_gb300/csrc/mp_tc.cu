@@ -72,11 +72,6 @@ struct TcDims {
     static constexpr uint32_t e_part = NB * E_BLK, e_bytes = 2 * e_part;
 };
 
-// A bounded wait with one answer for the warp.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
-    return __all_sync(DMTS_FULL, mbar_wait(bar, parity)) != 0;
-}
-
 // ---------------------------------------------------------------- front end
 // A CTA's work comes in chunks of up to 64 active edges of one receiver (the
 // g-th active edge of a row is slot g % 64 of chunk g / 64, whatever skin

@@ -81,6 +81,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
     return false;
 }
 
+// The same with one answer for the (converged) warp: where a warp-wide
+// instruction, such as a TMEM load, depends on it, a wait that runs out in some
+// lanes only must not split the warp.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity)) != 0;
+}
+
 // Orders earlier generic-proxy accesses to shared memory before later
 // asynchronous-proxy ones (a bulk copy that overwrites a buffer just read).
 __device__ __forceinline__ void fence_proxy_async_smem() {
