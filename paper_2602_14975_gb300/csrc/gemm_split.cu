@@ -18,7 +18,11 @@
 // against 252 us at 80 atoms), from 2,000 rows on slower (555 against 487 at
 // 3,000); one kernel serves every row count, so that an atom's bits do not
 // depend on its batch.
+//
+// Range: values from 2^-102 on keep 24 bits (below it the last part falls among
+// bf16's subnormals); a sum that is not finite is formed again in fp32.
 #include <algorithm>
+#include <cfloat>
 
 #include "epilogue.cuh"
 #include "launch.cuh"
@@ -66,6 +70,22 @@ __device__ __forceinline__ void store_split3(uint8_t *tile, uint32_t part, int r
 #pragma unroll
     for (int s = 0; s < 3; ++s)
         *reinterpret_cast<uint4 *>(tile + s * part + o) = make_uint4(p[s][0], p[s][1], p[s][2], p[s][3]);
+}
+
+// The sums of o (columns n0 .. of row m) that are not finite, once more in fp32
+// as the SIMT kernel forms them (even and odd k apart): parts of a value past
+// bf16's largest (3.39e38) or of an infinity are NaN, and parts may overflow
+// where their sum does not. 32 comparisons per thread where every sum is finite.
+__device__ __noinline__ void sums_again(float *o, int cols, int m, int n0, int M, int N, int K,
+                                        const float *__restrict__ Act, const float *__restrict__ W, int trans) {
+    if (m >= M) return;
+    for (int v = 0; v < cols && n0 + v < N; ++v) {
+        if (fabsf(o[v]) <= FLT_MAX) continue;
+        float s[2] = {0.f, 0.f};
+        for (int k = 0; k < K; ++k)
+            s[k & 1] = fmaf(Act[(size_t)m * K + k], trans ? W[(size_t)(n0 + v) * K + k] : W[(size_t)k * N + n0 + v], s[k & 1]);
+        o[v] = s[0] + s[1];
+    }
 }
 
 }  // namespace
@@ -222,6 +242,10 @@ __global__ void __launch_bounds__(TH, MINB) k_gemm_split(int M, int N, int K, co
         float *o = tile + (32 * (warp & 3) + lane) * D::LD + CW * (warp >> 2);
 #pragma unroll
         for (int v = 0; v < CW; ++v) o[v] = acc[v];
+        bool finite = true;
+#pragma unroll
+        for (int v = 0; v < CW; ++v) finite = finite && fabsf(acc[v]) <= FLT_MAX;
+        if (!finite) sums_again(o, CW, m0 + 32 * (warp & 3) + lane, n0 + CW * (warp >> 2), M, N, K, Act, W, trans);
         __syncthreads();
         const int rows = min(GS_BM, M - m0), cols = min(BN, N - n0);
         if (vec) epilogue_tile_v4(e, N, rows, m0, n0, cols, tile, D::LD);
