@@ -102,6 +102,28 @@ static bool upload(DevModel &m, const std::vector<float> &h) {
     return cudaMemcpy(m.dev, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
+// Channel scales of a tensor-core layer. Its features are split into fp16 pairs
+// under one power of two per row, so a channel far below its row's largest would
+// lose bits that may matter: s_c may be small because the weights that read it
+// are large. What a channel adds to the layer's MLP input goes as
+// (s_c wrad_lkc)^2 W1[o][l C + c], whatever the scale it is held in, so features
+// are split as s_c 2^g with 2^g the size of max_l max_k |wrad_lkc| sqrt(max_o |W1|),
+// and the sums are taken with wrad_lkc 2^-g; both are exact.
+static void tc_channel_scales(int C, int NL, int K, const float *wrad, const float *w1, float *scale, float *wrad_tc) {
+    for (int c = 0; c < C; ++c) {
+        double top = 0.0;
+        for (int l = 0; l < NL; ++l) {
+            double w = 0.0, u = 0.0;
+            for (int k = 0; k < K; ++k) w = std::max(w, (double)std::fabs(wrad[(l * K + k) * C + c]));
+            for (int o = 0; o < C; ++o) u = std::max(u, (double)std::fabs(w1[(size_t)o * NL * C + l * C + c]));
+            top = std::max(top, w * std::sqrt(u));
+        }
+        const int g = top > 0.0 && std::isfinite(top) ? std::min(std::max(std::ilogb(top), -100), 100) : 0;
+        scale[c] = top == 0.0 ? 0.f : std::ldexp(1.f, g);   // (a channel nothing reads sets no row's scale)
+        for (int q = 0; q < NL * K; ++q) wrad_tc[q * C + c] = std::ldexp(wrad[q * C + c], -g);
+    }
+}
+
 static dmts_status load_model(dmts_ctx *ctx, const dmts_model *in, bool is_nc, DevModel &m) {
     m.L = is_nc ? 1 : in->L;
     m.C = in->C;
@@ -142,6 +164,17 @@ static dmts_status load_model(dmts_ctx *ctx, const dmts_model *in, bool is_nc, D
         return fail(ctx, DMTS_E_INVALID, "weight blob size does not match the model sizes");
     std::vector<float> h(in->weights, in->weights + expect);
     if (is_nc) h.resize(expect + (size_t)m.nl * S * K);   // room for UW
+    const bool tc = !is_nc && m.bf16 && mp_tc_supported(C, K);
+    const size_t tc_len = (size_t)C + (size_t)NL * K * C;   // per layer after the first
+    if (tc) {
+        h.resize(expect + tc_len * (m.L - 1));
+        const size_t layer = (size_t)NL * K * C + (size_t)C * NL * C + C + (size_t)C * C + C;
+        for (int t = 1; t < m.L; ++t) {
+            const float *wrad = h.data() + (size_t)S * C + layer * t;
+            float *own = h.data() + expect + tc_len * (t - 1);
+            tc_channel_scales(C, NL, K, wrad, wrad + (size_t)NL * K * C, own, own + C);
+        }
+    }
     if (!upload(m, h)) return fail(ctx, DMTS_E_OOM, "weight upload failed");
     m.n_weights = (size_t)expect;
     // offsets (same order as the blob)
@@ -159,6 +192,10 @@ static dmts_status load_model(dmts_ctx *ctx, const dmts_model *in, bool is_nc, D
         m.wr = take((size_t)C * C);
         m.br = take(C);
         m.wo = take(C);
+        for (int t = 1; tc && t < m.L; ++t) {
+            m.ch_scale[t] = take(C);
+            m.wrad_tc[t] = take((size_t)NL * K * C);
+        }
     } else {
         const int H = K + m.nl;
         m.U = take((size_t)m.nl * C);
@@ -369,7 +406,8 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
                 io.s16 = (const __half *)w.s16.p;
                 io.s_exp = (const int *)w.s_exp.p;
                 io.q = nullptr;                 // the tensor-core contraction reads only the split-bf16 copy
-                launch_feature_split(N, io.s, (void *)io.s16, (int *)io.s_exp, st);
+                io.wrad = m.wrad_tc[t];
+                launch_feature_split(N, io.s, m.ch_scale[t], (void *)io.s16, (int *)io.s_exp, st);
                 launch_mp_fwd_tc(m.lmax, g, io, ctx->d_err, st);
             } else {
                 launch_mp_fwd(C, m.lmax, m.K, g, io, st);

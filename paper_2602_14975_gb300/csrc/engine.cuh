@@ -42,6 +42,9 @@ struct DevModel {
           *w2[DMTS_MAX_LAYERS] = {}, *b2[DMTS_MAX_LAYERS] = {};
     float *wr = nullptr, *br = nullptr, *wo = nullptr;
     float *U = nullptr, *Wqk = nullptr;
+    // tensor-core layers (tc_channel_scales): per channel a power of two for the
+    // features, [C], and the radial weights divided by it, [l_max + 1][K][C]
+    float *ch_scale[DMTS_MAX_LAYERS] = {}, *wrad_tc[DMTS_MAX_LAYERS] = {};
     float *UW = nullptr;                  // [n_l][S][K] of the first layer (launch_tensor_head_weights), after the blob
     // split-bf16 copies for the tensor-core contractions, every one K-major
     // ([out][2 in]: hi | lo): W1, W2, Wr (forward), their transposes

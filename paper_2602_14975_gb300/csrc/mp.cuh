@@ -110,11 +110,12 @@ void launch_first_bwd(int C, int lmax, const EdgeGeom &g, const FirstIO &io, cud
 void launch_mp_fwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io, cudaStream_t st);
 // The layers after the first on the tensor cores (mp_tc.cu; C = 128 and K = 8
 // only): the neighbour sums as products with split-fp16 operands. s16 and
-// s_exp hold the features' split copy ([N][2C] fp16 and one exponent per
-// row, launch_feature_split). err receives DMTS_E_TIMEOUT if a bounded wait
+// s_exp hold the split copy of the features times their channel's scale
+// ([N][2C] fp16 and one exponent per row, launch_feature_split); wrad is divided
+// by that scale. err receives DMTS_E_TIMEOUT if a bounded wait
 // on the tensor cores runs out.
 bool mp_tc_supported(int C, int K);
-void launch_feature_split(int n, const float *s, void *s16, int *s_exp, cudaStream_t st);
+void launch_feature_split(int n, const float *s, const float *ch_scale, void *s16, int *s_exp, cudaStream_t st);
 void launch_mp_fwd_tc(int lmax, const EdgeGeom &g, const LayerIO &io, int *err, cudaStream_t st);
 void launch_mp_bwd(int C, int lmax, int K, const EdgeGeom &g, const LayerIO &io, cudaStream_t st);
 // The adjoint's fixed-point forces (and virial, Wfix nullable) -> fp32 F and
