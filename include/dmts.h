@@ -50,8 +50,8 @@ typedef enum {
     DMTS_E_CUDA = 3,          /* a CUDA call failed */
     DMTS_E_NBR_OVERFLOW = 4,  /* neighbour list larger than its capacity */
     DMTS_E_NONFINITE = 5,     /* NaN/Inf found in positions or velocities */
-    DMTS_E_TIMEOUT = 6,       /* a bounded wait of a device kernel on its own asynchronous copies or
-                                 tensor-core work gave up; the context stays usable */
+    DMTS_E_TIMEOUT = 6,       /* a bounded wait of a device kernel on its own asynchronous copies,
+                                 tensor-core work or other blocks gave up; the context stays usable */
     DMTS_E_BUSY = 7           /* state already in use by an unfinished call */
 } dmts_status;
 
@@ -549,6 +549,15 @@ dmts_status dmts_contract_bf16(dmts_ctx *ctx, int M, int N, int K, const void *a
  * next dmts_sync() returns DMTS_E_TIMEOUT (and clears it) and the context
  * stays usable. limit_us in [1, 1000000], else DMTS_E_INVALID. */
 dmts_status dmts_check_bounded_wait(dmts_ctx *ctx, int limit_us, void *stream);
+
+/* (No counterpart in the paper: failure detection.) The same for the barrier
+ * over the grid that a state's list rebuild passes between its phases (limit
+ * there: 10 s): one launch of two blocks that meet at it with a limit of
+ * limit_us, or, with absent = 0 or 1, of which that block never comes. The
+ * other's wait then runs out (after twice limit_us where block 0 is absent)
+ * and dmts_sync() returns DMTS_E_TIMEOUT once; with absent = -1 it returns
+ * DMTS_OK. limit_us in [1, 1000000], else DMTS_E_INVALID. */
+dmts_status dmts_check_bounded_barrier(dmts_ctx *ctx, int limit_us, int absent, void *stream);
 
 /* Bytes of device workspace a replica of n_atoms needs in the serving loop
  * (admission accounting). */

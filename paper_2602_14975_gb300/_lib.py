@@ -105,7 +105,8 @@ EXPORTS = ("dmts_create", "dmts_destroy", "dmts_last_error", "dmts_sync", "nbr_b
            "energy_forces_cons", "forces_nc", "respa_step", "dmts_state_release", "dmts_state_lists", "nc_distill_step", "run_replicas",
            "dmts_masses_hmr", "dmts_bond_table", "dmts_philox_words", "dmts_gaussians",
            "dmts_replica_footprint", "dmts_profile_enable", "dmts_profile_read", "nbr_build_noalloc",
-           "dmts_contract_bf16", "dmts_kernel_launches", "respa_guarded", "dmts_check_bounded_wait")
+           "dmts_contract_bf16", "dmts_kernel_launches", "respa_guarded", "dmts_check_bounded_wait",
+           "dmts_check_bounded_barrier")
 
 
 def lib_path() -> str:
@@ -159,6 +160,8 @@ def _declare(L):
     L.dmts_contract_bf16.argtypes = [vp, i, i, i, vp, vp, vp, i, vp]
     L.dmts_check_bounded_wait.restype = i
     L.dmts_check_bounded_wait.argtypes = [vp, i, vp]
+    L.dmts_check_bounded_barrier.restype = i
+    L.dmts_check_bounded_barrier.argtypes = [vp, i, i, vp]
     L.nbr_build_noalloc.restype = i
     L.nbr_build_noalloc.argtypes = [ct.POINTER(System), ct.POINTER(Nbr), ct.POINTER(ct.c_longlong), vp]
     L.dmts_profile_enable.restype = i

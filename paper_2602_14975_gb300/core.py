@@ -470,3 +470,11 @@ def check_bounded_wait(ctx: Context, limit_us: int) -> int:
     (DMTS_E_TIMEOUT expected); the sticky error word is cleared."""
     L.check(ctx.lib.dmts_check_bounded_wait(ctx.handle, int(limit_us), _stream()), ctx.handle)
     return int(ctx.lib.dmts_sync(ctx.handle, _stream()))
+
+
+def check_bounded_barrier(ctx: Context, limit_us: int, absent: int) -> int:
+    """Runs the list rebuild's barrier over two blocks, of which block `absent`
+    (0 or 1; -1: none) never comes, and returns the status dmts_sync then
+    reports (DMTS_E_TIMEOUT expected; DMTS_OK with -1)."""
+    L.check(ctx.lib.dmts_check_bounded_barrier(ctx.handle, int(limit_us), int(absent), _stream()), ctx.handle)
+    return int(ctx.lib.dmts_sync(ctx.handle, _stream()))

@@ -1835,6 +1835,16 @@ dmts_status dmts_check_bounded_wait(dmts_ctx *ctx, int limit_us, void *stream) {
     return ck(ctx, cudaGetLastError(), "dmts_check_bounded_wait launch") ? DMTS_OK : DMTS_E_CUDA;
 }
 
+dmts_status dmts_check_bounded_barrier(dmts_ctx *ctx, int limit_us, int absent, void *stream) {
+    if (!ctx || limit_us < 1 || limit_us > 1000000 || absent < -1 || absent > 1)
+        return fail(ctx, DMTS_E_INVALID, "dmts_check_bounded_barrier: limit_us in [1, 1000000], absent in -1..1");
+    cudaSetDevice(ctx->device);
+    Buf &b = ctx->nbr_scratch.sync;
+    if (!b.ensure(4 * sizeof(unsigned))) return fail(ctx, DMTS_E_OOM, "barrier words");
+    nbr_check_barrier((unsigned *)b.p, absent, (uint64_t)limit_us * 1000ull, ctx->d_err, (cudaStream_t)stream);
+    return ck(ctx, cudaGetLastError(), "dmts_check_bounded_barrier launch") ? DMTS_OK : DMTS_E_CUDA;
+}
+
 __global__ void k_philox_words(uint64_t seed, uint32_t rep, uint64_t step, uint32_t atom0, int count, uint32_t *out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;

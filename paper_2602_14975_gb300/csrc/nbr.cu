@@ -725,14 +725,17 @@ void nbr_fill(const NbrWork &w, float r_list, int *row_ptr, int *col, long long 
 // ----------------------------------------------------------- gated rebuild
 // A state's rebuild as one cooperative launch: the phases above with barriers
 // over the grid between them. Every inner step asks for one and most find the
-// gate closed; as eight launches (cells, scans, count, fill, gate) that cost
-// XX.
+// gate closed; as eight launches (cells, scans, count, fill, gate) an outer step
+// of 192 atoms took 223 us, as one 212.
 //
 // Barrier: block b > 0 writes the epoch (launch number, phase) to its word and
 // waits for block 0's release word; block 0 collects the words, reads the
 // error word once for everybody and releases with a stop bit. Every wait is
-// bounded, by more than a long kernel of another stream can keep the last
-// blocks from starting; words of an earlier launch never match.
+// bounded twice, as the mbarrier waits are (ptx.cuh): by 10 s, 20 s for the
+// blocks that wait for block 0, which is more than a long kernel of another
+// stream can keep the last blocks from starting, and by a poll count. A wait
+// that runs out records DMTS_E_TIMEOUT and every block leaves. Words of an
+// earlier launch never match.
 constexpr int RB_THREADS = NBC_WARPS * 32;
 constexpr uint64_t RB_WAIT_NS = 10 * kWaitLimitNs;
 static_assert(RB_THREADS == SCAN_THREADS, "one block shape for every phase");
@@ -746,18 +749,32 @@ __device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Polls *p until *p >> shift is `want`; false once limit_ns have passed or
+// kSpinLimit polls were made. v: the word last read.
+__device__ __forceinline__ bool poll_word(const unsigned *p, int shift, unsigned want, uint64_t limit_ns, unsigned &v) {
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; it < kSpinLimit; ++it) {
+        v = ld_acquire(p);
+        if (v >> shift == want) return true;
+        if ((it & 15u) == 0) {
+            const uint64_t t = globaltimer_ns();
+            if (it == 0) t0 = t;
+            else if (t - t0 > limit_ns) return false;
+        }
+    }
+    return false;
+}
+
 // False: a stop (error recorded, or a block that never came).
-__device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned epoch, int *err) {
+__device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned epoch, int *err, uint64_t limit_ns = RB_WAIT_NS) {
     __shared__ int go;
     unsigned *release = sync + 1, *words = sync + 2;
     __syncthreads();
     if (blockIdx.x == 0) {
         int ok = 1;
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-            const uint64_t t0 = globaltimer_ns();
-            while (b > 0 && ok && ld_acquire(words + b) != epoch)
-                if (globaltimer_ns() - t0 > RB_WAIT_NS) ok = 0;
-        }
+        unsigned v;
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
+            if (b > 0 && ok) ok = poll_word(words + b, 0, epoch, limit_ns, v);
         ok = __syncthreads_and(ok);
         if (threadIdx.x == 0) {
             if (!ok) set_error(err, DMTS_E_TIMEOUT);
@@ -768,11 +785,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned epoch, int
     } else if (threadIdx.x == 0) {
         __threadfence();
         st_release(words + blockIdx.x, epoch);
-        const uint64_t t0 = globaltimer_ns();
         unsigned v;
-        bool ok = true;
-        while (((v = ld_acquire(release)) >> 1) != epoch && ok)
-            if (globaltimer_ns() - t0 > 2 * RB_WAIT_NS) ok = false;
+        const bool ok = poll_word(release, 1, epoch, 2 * limit_ns, v);
         if (!ok) set_error(err, DMTS_E_TIMEOUT);
         go = ok && !(v & 1u);
         __threadfence();
@@ -869,6 +883,26 @@ void nbr_rebuild(const NbrWork &w, float r_list, int *row_ptr, int *col, long lo
     cfg.attrs = at;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, k_nbr_rebuild, wc, a);
+    count_launch();
+}
+
+// The barrier over two blocks, of which block `absent` (none if < 0) never comes.
+__global__ void __launch_bounds__(RB_THREADS) k_check_barrier(unsigned *sync, int absent, uint64_t limit_ns, int *err) {
+    if ((int)blockIdx.x != absent) grid_barrier(sync, 8, err, limit_ns);
+}
+
+void nbr_check_barrier(unsigned *sync, int absent, uint64_t limit_ns, int *err, cudaStream_t st) {
+    cudaMemsetAsync(sync, 0, 4 * sizeof(unsigned), st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3(RB_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_check_barrier, sync, absent, limit_ns, err);
     count_launch();
 }
 

@@ -69,6 +69,9 @@ constexpr int kRebuildBlocks = 1024;
 void nbr_rebuild(const NbrWork &w, float r_list, int *row_ptr, int *col, long long capacity, float *x_ref,
                  unsigned *sync, int *gate, cudaStream_t st, float r_sub = 0.f, int *sub_row = nullptr,
                  int *sub_col = nullptr, long long sub_capacity = -1);
+// Its barrier alone, over two blocks with a limit of its own (sync: 4 words):
+// the waits run out if block `absent` is 0 or 1, and pass if it is negative.
+void nbr_check_barrier(unsigned *sync, int absent, uint64_t limit_ns, int *err, cudaStream_t st);
 // Atom -> replica map.
 void atom_rep_map(const int *rep_off, int n_rep, int n_atoms, int *atom_rep, cudaStream_t st);
 // Exclusive scans of n ints into out[n+1], one or two arrays in one launch
