@@ -353,7 +353,7 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
     Workspace &w = ctx->ws;
     const size_t nc_ = (size_t)N * C;
     const bool bf = m.bf16;
-    if (!w.s.ensure(sizeof(float) * nc_ * (L + 1)) || !w.A.ensure(sizeof(float) * nc_ * NLM * L) ||
+    if (!w.s.ensure(sizeof(float) * nc_ * L) || !w.A.ensure(sizeof(float) * nc_ * NLM * L) ||
         !w.q.ensure(sizeof(float) * nc_ * NL) || !w.h.ensure(sizeof(float) * nc_ * L) ||
         !w.act.ensure(sizeof(float) * nc_) || !w.u.ensure(sizeof(float) * nc_) || !w.gz.ensure(sizeof(float) * nc_) ||
         !w.gs0.ensure(sizeof(float) * nc_) || !w.gs1.ensure(sizeof(float) * nc_) ||
@@ -375,7 +375,9 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
     if (bf && (!w.q_bf.ensure(4 * nc_ * NL + 16) || !w.act_bf.ensure(4 * nc_ + 16) || !w.s_bf.ensure(4 * nc_ + 16) ||
                !w.gz_bf.ensure(4 * nc_ + 16) || !w.gs0_bf.ensure(4 * nc_ + 16) || !w.gs1_bf.ensure(4 * nc_ + 16)))
         return fail(ctx, DMTS_E_OOM, "workspace allocation failed");
-    float *S = (float *)w.s.p, *A = (float *)w.A.p, *q = (float *)w.q.p, *H = (float *)w.h.p;
+    // features s^t of layer t >= 1 (and the readout's, t = L); s^0 is the species embedding
+    auto S = [&](int t) { return (float *)w.s.p + nc_ * (t - 1); };
+    float *A = (float *)w.A.p, *q = (float *)w.q.p, *H = (float *)w.h.p;
     float *act = (float *)w.act.p, *u = (float *)w.u.p, *gz = (float *)w.gz.p;
     float *gs0 = (float *)w.gs0.p, *gs1 = (float *)w.gs1.p, *gA = (float *)w.gA.p;
     float *e_atom = (float *)w.e_atom.p;
@@ -386,7 +388,7 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
     for (int t = 0; t < L; ++t) {
         LayerIO io;
         memset(&io, 0, sizeof io);
-        io.s = S + nc_ * t;
+        io.s = t == 0 ? nullptr : S(t);
         io.wrad = m.wrad[t];
         io.nu = m.nu;
         io.A = A + nc_ * NLM * t;
@@ -422,9 +424,9 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
             return DMTS_E_CUDA;
         Epi e2 = epi(EPI_RESID);
         e2.bias = m.b2[t];
-        e2.res = t == 0 ? m.emb : S + nc_ * t;   // s^0 is the species embedding
+        e2.res = t == 0 ? m.emb : S(t);
         e2.res_row = t == 0 ? s.species : nullptr;
-        e2.out = S + nc_ * (t + 1);
+        e2.out = S(t + 1);
         e2.out_bf16 = t == L - 1 ? s_bf : nullptr;
         if (!contract(ctx, m, N, C, C, act, act_bf, m.w2[t], 1, m.w2_bf[t], e2, st, "gemm_tc", "gemm"))
             return DMTS_E_CUDA;
@@ -436,7 +438,7 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
     er.out = u;
     er.out2 = gz;
     er.out_bf16 = gz_bf;
-    if (!contract(ctx, m, N, C, C, S + nc_ * L, s_bf, m.wr, 1, m.wr_bf, er, st, "gemm_tc", "gemm"))
+    if (!contract(ctx, m, N, C, C, S(L), s_bf, m.wr, 1, m.wr_bf, er, st, "gemm_tc", "gemm"))
         return DMTS_E_CUDA;
     { ProfScope ps(ctx, "rowsum", st); launch_rowsum(N, C, u, m.scale, e_atom, st); }
     if (forces) {
@@ -479,7 +481,7 @@ dmts_status cons_eval(dmts_ctx *ctx, const SysView &s, const int *row_ptr, const
                 return DMTS_E_CUDA;
             LayerIO io;
             memset(&io, 0, sizeof io);
-            io.s = S + nc_ * t;
+            io.s = S(t);
             io.wrad = m.wrad[t];
             io.nu = m.nu;
             io.gA = gA;
