@@ -150,14 +150,18 @@ long long dmts_replica_footprint(const dmts_ctx *ctx, int n_atoms) {
     // neighbour lists (about 80 + 40 entries per atom with head-room) and the
     // sorted rows kept between the count and the fill of a rebuild
     b += (long long)n_atoms * 4 * (160 + kNbrSlots);
-    // activations of the conservative model
+    // the conservative evaluation (cons_eval): [N][C] arrays of 4-byte elements
+    // (features, A, q, pre-activations, five MLP and gradient arrays, gA), and
+    // one more for its words per atom (energy, forces, fixed-point sums)
     const DevModel &m = ctx->cons;
-    const int nlm = (m.lmax + 1) * (m.lmax + 1);
-    b += (long long)n_atoms * m.C * 4 * (m.L + 1 + m.L * nlm + (m.lmax + 1) + m.L + 6 + nlm);
-    // split-bf16 operand copies (hi and lo: 4 bytes per element) of q and of
-    // the five [N][C] contraction inputs
-    if (m.bf16) b += (long long)n_atoms * m.C * 4 * ((m.lmax + 1) + 5);
-    return b;
+    const int nl = m.lmax + 1, nlm = nl * nl;
+    int arrays = m.L + m.L * nlm + nl + m.L + 5 + (m.L > 1 ? nlm : 0) + 1;
+    // split-bf16 operand copies (hi and lo) of q and of the five contraction inputs
+    if (m.bf16) arrays += nl + 5;
+    // the tensor-core layers' split-fp16 features (and a row exponent each)
+    const bool tc = m.bf16 && m.L > 1 && mp_tc_supported(m.C, m.K);
+    if (tc) arrays += 1;
+    return b + (long long)n_atoms * 4 * ((long long)m.C * arrays + tc);
 }
 
 dmts_status run_replicas(dmts_ctx *ctx, const dmts_request *reqs, int n_req, const dmts_integrator *p,

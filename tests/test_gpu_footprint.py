@@ -53,3 +53,15 @@ def test_features_of_the_layers_only():
     n, C = 1_000_000, 128
     taken, _ = growth(S.cons_spec(1, C, 0), n)
     assert taken <= n * (4 * C * 9 + 44) + ROUNDING
+
+
+@pytest.mark.parametrize("C,L,lmax,bf16", [(128, 3, 2, True), (128, 1, 1, True), (64, 2, 1, True), (128, 2, 0, False)])
+def test_admission_counts_what_is_allocated(C, L, lmax, bf16):
+    """The serving loop's count per replica, less its share of state and lists
+    (85 bytes and 288 list words per atom), covers what an evaluation takes and
+    exceeds it by no more than the one array it allows for words per atom."""
+    n = 1_000_000
+    taken, fp = growth(S.cons_spec(L, C, lmax, bf16=bf16), n)
+    counted = fp - n * (85 + 4 * 288)
+    assert taken <= counted + ROUNDING
+    assert counted <= taken + n * 4 * C + ROUNDING
