@@ -329,6 +329,49 @@ def integ_bytes_per_outer_step(n_inner, with_close):
     return INTEG_B_KICK + INTEG_B_INNER * (n_inner - 1) + (INTEG_B_CLOSE if with_close else 0)
 
 
+def kernel_work(cs, ns):
+    """What the message-passing kernels execute and move per launch, as
+    {kernel: {"edge": FLOP per active directed edge, "atom": FLOP per atom,
+    "tensor_edge": those of the edge's on the tensor cores, "bytes_atom": bytes
+    per atom, each array once}} (an FMA is 2 FLOP; edge geometry, radial functions
+    and harmonics are not counted; 4 bytes of column index per edge besides).
+
+    first_fwd / first_bwd: the first layer, factored over species: basis sums of
+    K (l_max+1)^2 products per edge, and per atom their contraction with the
+    weights, counted for every species (fewer occur around most atoms).
+    mp_fwd / mp_bwd: one of the L - 1 later layers. On the tensor cores (split
+    bf16, C = 128) the neighbour sum is a dense product of the padded (l, m, k)
+    columns, three fp16 products each, and the radial weights are applied per
+    atom; else 36 FMA per edge and channel at l_max = 2. The adjoint forms each
+    pair once, from its lower atom (at l_max = 2 99 FMA per channel, 51 FLOP per
+    lane for the direction derivative, 93 adds for the lanes' sums), and the
+    lower atom's sender-role term of the reverse edge takes 36 per channel: a
+    directed edge averages half of both."""
+    out = {}
+    for k, m, lmax in (("first_fwd", cs, cs.lmax), ("nc_mp_fwd", ns, 1)):
+        nl, S, K, C = lmax + 1, m.n_species, m.K, m.C
+        nlm = nl * nl
+        out[k] = {"edge": 2 * K * nlm, "atom": 2 * S * (K + 1) * nlm * C + 3 * nlm * C, "tensor_edge": 0,
+                  "bytes_atom": 12 + 1 + 4 * nl * C + (4 * nlm * C if k == "first_fwd" else 4 * 3 * m.n_l)}
+    nl, S, K, C = cs.lmax + 1, cs.n_species, cs.K, cs.C
+    nlm = nl * nl
+    out["first_bwd"] = {"edge": 2 * K * (2 * nlm - 1) + 2 * (4 * nlm - 3), "tensor_edge": 0,
+                        "atom": 2 * S * K * C * (nlm + nl / 2) + 2 * nlm * C,
+                        "bytes_atom": 12 + 1 + 4 * nl * C + 4 * nlm * C + 48}
+    tc = cs.bf16 and C == 128 and K == 8
+    if tc:
+        cols = 16 * ((nlm * K + 15) // 16)
+        out["mp_fwd"] = {"edge": 2 * 3 * cols * C, "tensor_edge": 2 * 3 * cols * C, "atom": 2 * nlm * K * C + 3 * nlm * C,
+                         "bytes_atom": 12 + 4 + 4 * C + 4 * nlm * C + 4 * nl * C}
+    else:
+        out["mp_fwd"] = {"edge": 2 * (K * nl + nlm + nl) * C, "tensor_edge": 0, "atom": 3 * nlm * C,
+                         "bytes_atom": 12 + 4 * C + 4 * nlm * C + (8 if cs.bf16 else 4) * nl * C}
+    pair, lower = 2 * K * nl + 5 * nlm + 2 * nl, K * nl + nlm + nl        # FMA per channel: 99 and 36 at l_max = 2
+    out["mp_bwd"] = {"edge": (pair + lower) * C + 51 * 32 / 2 + 93 / 2, "tensor_edge": 0, "atom": 4 * C,
+                     "bytes_atom": 12 + 4 * C + 4 * nlm * C + 4 * C + (8 if cs.bf16 else 4) * C + 48}
+    return out
+
+
 def serving_roofline(prof, atom_outer_steps, n_inner, cs):
     """Per-kernel rates inside the serving loop, where one launch covers every
     resident replica (often 10^5 atoms or more): the integrator against HBM
@@ -839,50 +882,32 @@ def main():
     Lc = cs.L
     nl1 = cs.lmax + 1
     nlm = nl1 * nl1
-    # the method's work per active edge and layer (each FMA 2 FLOP): the
-    # radial contraction R_lc = sum_k W B_k (K (l_max+1) FMA per channel) and
-    # the message into A_lm (one FMA per (l, m) and channel); the adjoint
-    # with per-layer recomputation counts twice the forward
-    flop_method = {"mp_fwd": 2 * (cs.K * nl1 + nlm) * C}
-    flop_method["mp_bwd"] = 2 * flop_method["mp_fwd"]
-    # what the kernels execute per active edge (each FMA 2 FLOP): forward
-    # 36 FMA per channel; the adjoint forms each pair once, from its lower
-    # atom: 99 FMA per channel (87 in layer 0, which has no sender-role
-    # gradient), 30 per lane for the direction derivatives and 93 adds for
-    # the lanes' sum of the pair force, and the lower atom's sender-role
-    # term of the reverse edge takes 36 per channel (none in layer 0), so a
-    # directed edge averages half of a pair; averaged over the L launches of
-    # one evaluation
-    flop_kernel = {"mp_fwd": 2 * 36 * C,
-                   "mp_bwd": ((99 + 36) * C * (Lc - 1) + 87 * C) / Lc + 30 * 32 + 93 / 2}
-    # a split-bf16 model with C = 128 runs the forward's radial contraction
-    # on the tensor cores (three bf16 MMAs per product, K = 8): 12 FMA per
-    # channel stay on the CUDA cores
-    fwd_tc = cs.bf16 and C == 128 and cs.K == 8
-    if fwd_tc:
-        flop_kernel["mp_fwd"] = 2 * (nlm + nl1) * C
-        flop_tensor_fwd = 2 * 3 * cs.K * nl1 * C
+    # the method's work per active edge of a later layer's adjoint (each FMA 2
+    # FLOP): twice the forward's radial contraction R_lc = sum_k W B_k (K (l_max+1)
+    # FMA per channel) and message into A_lm (one FMA per (l, m) and channel), as
+    # every edge quantity is recomputed
+    flop_method = 2 * 2 * (cs.K * nl1 + nlm) * C
+    work = kernel_work(cs, ns)
 
     def per_launch_s(pr, k):
         v = pr.get(k)
         return v[1] / v[0] * 1e-3 if v and v[0] else None
 
-    ranked = sorted(((k, v) for k, v in prof.items() if k in flop_method), key=lambda kv: -kv[1][1])
-    name = ranked[0][0] if ranked else "mp_bwd"
+    name = "mp_bwd"              # the dominant kernel: every layer but the first
     pl = per_launch_s(prof, name)
-    achieved = flop_method[name] * e_cons / pl / 1e12 if pl else None
-    # node arrays once and the active-edge stream (4 B of column index per
-    # active entry): forward reads s, x and writes A, q (+ its split-bf16
-    # copy); the adjoint reads s, gA, g_s and x and writes g_s (+ copy) and F
+    achieved = flop_method * e_cons / pl / 1e12 if pl else None
     n_at = sy.n_atoms
-    alg_bytes = {"mp_fwd": n_at * (4 * C + 12 + 4 * nlm * C + 8 * nl1 * C) + 4 * e_cons,
-                 "mp_bwd": n_at * (4 * C + 4 * nlm * C + 12 + 12 + (Lc - 1) / Lc * (4 * C + 8 * C)) + 4 * e_cons}
+
+    def executed(k, edges):
+        return work[k]["edge"] * edges + work[k]["atom"] * n_at
+
     roof = {"kernel": name, "bound": "alu", "achieved": achieved, "peak": fp32_pk, "unit": "TFLOP/s",
             "frac": achieved / fp32_pk if achieved else None, "traffic": ncu_traffic(name),
-            "work": f"{flop_method[name]} FLOP per active edge (the method's count) x {e_cons} edges per launch",
+            "work": f"{flop_method} FLOP per active edge (the method's count) x {e_cons} edges per launch, one of "
+                    f"{Lc - 1} layers",
             "peak_source": fp32_src,
-            "kernel_executed_tflops": flop_kernel[name] * e_cons / pl / 1e12 if pl else None,
-            "algorithmic_bytes_per_launch": alg_bytes[name]}
+            "kernel_executed_tflops": executed(name, e_cons) / pl / 1e12 if pl else None,
+            "algorithmic_bytes_per_launch": work[name]["bytes_atom"] * n_at + 4 * e_cons}
 
     # every hot kernel against its own bound (per-launch averages over the
     # timed region; algorithmic work counts each node array once and each
@@ -901,16 +926,28 @@ def main():
     t_ncg = prof.get("nc_gemm_tc", (0, 0.0))[1] * 1e-3 / n_prof
     nc_bytes = N * (qkw * 4 + ns.n_l * 12 + 12 + 12) + 4 * e_nc
     kr = {}
-    for k in ("mp_fwd", "mp_bwd"):
-        a = rate(flop_method[k] * e_cons, per_launch_s(prof, k), 1e12)
-        kr[k] = {"row": "a2+a3" if k == "mp_fwd" else "a5", "bound": "alu", "tflops": a,
-                 "frac_fp32_peak": a / fp32_pk if a else None,
-                 "kernel_executed_tflops": rate(flop_kernel[k] * e_cons, per_launch_s(prof, k), 1e12)}
-    if fwd_tc:
-        kr["mp_fwd"]["bound"] = "latency (neighbour gathers)"
-        kr["mp_fwd"]["radial_on_tensor_cores_tflops"] = rate(flop_tensor_fwd * e_cons, per_launch_s(prof, "mp_fwd"), 1e12)
-        kr["mp_fwd"]["note"] = ("the method's count over the FP32 peak; the radial contraction runs on the tensor "
-                                "cores (three bf16 MMAs per product), the messages on the CUDA cores")
+    rows = {"first_fwd": ("a2+a3 (first layer)", "latency and shared-memory wavefronts", e_cons),
+            "first_bwd": ("a5 (first layer)", "latency and shared-memory wavefronts", e_cons),
+            "mp_fwd": ("a2+a3", "alu", e_cons), "mp_bwd": ("a5", "alu", e_cons),
+            "nc_mp_fwd": ("a7 (NC layer: a2+a3 at NC sizes, factored over species)",
+                          "latency and shared-memory wavefronts", e_nc)}
+    for k, (row, bound, edges) in rows.items():
+        t = per_launch_s(prof, k)
+        a, b = rate(executed(k, edges), t, 1e12), rate(work[k]["bytes_atom"] * n_at + 4 * edges, t, 1e9)
+        kr[k] = {"row": row, "bound": bound, "executed_flop_per_edge": work[k]["edge"],
+                 "executed_flop_per_atom": work[k]["atom"], "executed_tflops": a,
+                 "frac_fp32_peak": a / fp32_pk if a else None, "gbs": b, "frac_hbm": b / hbm if b and hbm else None}
+    kr["mp_bwd"]["method_tflops"] = achieved
+    if work["mp_fwd"]["tensor_edge"]:
+        a = rate(work["mp_fwd"]["tensor_edge"] * e_cons, per_launch_s(prof, "mp_fwd"), 1e12)
+        kr["mp_fwd"].update(bound="latency of a chunk's phases", frac_fp32_peak=None, tensor_tflops=a,
+                            frac_bf16_sustained=a / bf16_pk if a and bf16_pk else None,
+                            note="with the features' split before it; the whole neighbour sum runs on the tensor "
+                                 "cores (three fp16 products of the padded columns), the radial weights once per atom")
+    if "nbr_rebuild" in prof:
+        kr["nbr_rebuild"] = {"row": "a1", "bound": "latency", "launches_per_step": prof["nbr_rebuild"][0] / n_prof,
+                             "ms_per_step": prof["nbr_rebuild"][1] / n_prof,
+                             "note": "asked for every inner step; most launches find the gate closed"}
     g = rate(gemm_flop_cons, t_gemm, 1e12)
     kr["gemm_tc"] = {"row": "a4", "bound": "tensor", "tflops": g, "frac_bf16_sustained": g / bf16_pk if g and bf16_pk else None,
                      "flop_per_step": gemm_flop_cons,
@@ -918,11 +955,6 @@ def main():
     g = rate(gemm_flop_nc * I.n_inner, t_ncg, 1e12)
     kr["nc_gemm_tc"] = {"row": "a4 (NC)", "bound": "tensor", "tflops": g,
                         "frac_bf16_sustained": g / bf16_pk if g and bf16_pk else None}
-    nnl = ns.lmax + 1
-    flop_nc_edge = 2 * (ns.K * nnl + nnl + nnl * nnl) * Cn
-    a = rate(flop_nc_edge * e_nc, per_launch_s(prof, "nc_mp_fwd"), 1e12)
-    kr["nc_mp_fwd"] = {"row": "a7 (NC layer: a2+a3 at NC sizes)", "bound": "alu", "tflops": a,
-                       "frac_fp32_peak": a / fp32_pk if a else None, "flop_per_edge": flop_nc_edge}
     b = rate(nc_bytes, per_launch_s(prof, "nc_head"), 1e9)
     kr["nc_head"] = {"row": "a7", "bound": "hbm", "gbs": b, "frac_hbm": b / hbm if b and hbm else None,
                      "bytes_per_launch": nc_bytes}
