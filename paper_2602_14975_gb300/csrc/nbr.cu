@@ -752,15 +752,11 @@ __device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
 // Polls *p until *p >> shift is `want`; false once limit_ns have passed or
 // kSpinLimit polls were made. v: the word last read.
 __device__ __forceinline__ bool poll_word(const unsigned *p, int shift, unsigned want, uint64_t limit_ns, unsigned &v) {
-    uint64_t t0 = 0;
+    const uint64_t t0 = globaltimer_ns();
     for (uint32_t it = 0; it < kSpinLimit; ++it) {
         v = ld_acquire(p);
         if (v >> shift == want) return true;
-        if ((it & 15u) == 0) {
-            const uint64_t t = globaltimer_ns();
-            if (it == 0) t0 = t;
-            else if (t - t0 > limit_ns) return false;
-        }
+        if (globaltimer_ns() - t0 > limit_ns) return false;   // (also the pace of the polls)
     }
     return false;
 }
