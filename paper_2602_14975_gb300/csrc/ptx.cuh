@@ -35,11 +35,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Named barrier `id` (1..15) over `n` threads (whole warps), alone and with an
-// AND of a predicate.
-__device__ __forceinline__ void bar_sync(int id, int n) {
-    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
+// Named barrier `id` (1..15) over `n` threads (whole warps), with an AND of a
+// predicate.
 __device__ __forceinline__ bool bar_sync_and(int id, int n, bool v) {
     uint32_t r;
     asm volatile(
