@@ -57,7 +57,14 @@ typedef enum {
 
 /*
  * Arithmetic of the MLP contractions (the paper states none; the stand-in
- * models run them as follows). DMTS_FP32: fp32 SIMT products. DMTS_BF16:
+ * models run them as follows). DMTS_FP32: fp32 accuracy. Models of fewer than
+ * 128 channels: fp32 SIMT products. From 128 channels on: tensor cores, each
+ * operand held in three bf16 parts (24 significant bits for magnitudes from
+ * 2^-102 on), the six products down to 2^-16 of the largest accumulated in
+ * fp32, every 64 terms added to an fp32 sum (against 64 bits the forces' error
+ * is that of the SIMT products); a sum that is not finite is formed again in
+ * fp32. nc_distill_step's gradient contractions use the three-part products
+ * from 8,192 atoms and 64 channels on, whatever the precision. DMTS_BF16:
  * tensor cores, bf16 x bf16 products accumulated in fp32, each operand held
  * as a split pair hi = rn_bf16(v), lo = rn_bf16(v - hi) and the products
  * hi*hi + lo*hi + hi*lo accumulated (about 16 significant bits per operand;
@@ -185,7 +192,10 @@ dmts_status dmts_sync(dmts_ctx *ctx, void *stream);
  * the list cutoff nbr->r_list. Synchronous: *n_pairs receives the number of
  * stored pairs; if it exceeds nbr->capacity, col is left unspecified and
  * DMTS_E_NBR_OVERFLOW is returned (retry with capacity >= *n_pairs).
- * Periodic boxes need r_list < box/2 on every periodic axis.
+ * Periodic boxes need r_list < box/2 on every periodic axis. The context keeps
+ * the build's scratch for the next one, until dmts_destroy: up to 2^21 atoms
+ * (1 GiB) 512 bytes per atom for the sorted rows, without which larger systems,
+ * and systems for which that cannot be had, are built.
  */
 dmts_status nbr_build(dmts_ctx *ctx, const dmts_system *sys, dmts_nbr *nbr,
                       long long *n_pairs, void *stream);

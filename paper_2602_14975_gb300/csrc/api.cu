@@ -339,7 +339,10 @@ static bool contract(dmts_ctx *ctx, const DevModel &m, int M, int N, int K, cons
     }
     ProfScope ps(ctx, tag_f32, st);
     // (23,558 rows, C = 128: the 14 contractions of a conservative call 777 us
-    // SIMT, 510 split; at 192 rows of C = 64 7.4 us a call SIMT, 11.1 split)
+    // SIMT, 510 split. The line is by channels, not rows, so that an atom's bits
+    // do not depend on its batch; models of 64 channels are those of the smallest
+    // systems. Their force call, two layers, l_max = 1, SIMT | split: 192 atoms
+    // 101 | 118 us, 3,000 158 | 157, 12,288 383 | 359, 99,999 2,541 | 2,379)
     if (std::min(N, K) >= 128) launch_gemm_split(M, N, K, A32, W32, trans, e, ctx->d_err, st);
     else launch_gemm_f32(M, N, K, A32, W32, trans, e, st);
     return true;
