@@ -466,6 +466,13 @@ __device__ __forceinline__ void count_cell(const NbrWork &w, float rc2, float rc
         acc.finish(w, keep, i, lane);
     }
 }
+// MORE_L1: the same code with a carve-out for four blocks per SM; that for a fifth
+// leaves 28 instead of 60 KB of L1. It serves neighbourhoods that are not staged
+// (3,000 atoms, 259 neighbours each: hit rate 99.7 against 95.5 %, 620 us against
+// 1,020) and grids of few cells (20,000 atoms, 200 neighbours each, 343 cells: a
+// build 465 us against 495); beyond four blocks per SM the fifth is worth 1 us
+// (729 cells of water, count 36 us).
+template <bool MORE_L1>
 __global__ void __launch_bounds__(NBC_WARPS * 32) k_nbr_count_cell(NbrWork w, float rc2, float rc2_sub) {
     dep_entry();
     __shared__ CountSmem sm;
@@ -709,13 +716,28 @@ void nbr_fill(const NbrWork &w, float r_list, int *row_ptr, int *col, long long 
     const int nb = (w.n_atoms + NB_WARPS - 1) / NB_WARPS;
     NbrWork wc = w;
     if (!sub_row) wc.counts_sub = nullptr;
-    launch_dep(k_nbr_count_cell, wc.n_cells, NBC_WARPS * 32, 0, st, wc, r_list * r_list, r_sub * r_sub);
+    // more L1 where the grid has no use for a fifth block per SM, and where
+    // neighbourhoods are on average too large to stage
+    if (wc.n_cells <= 4 * sm_count() ||
+        (long long)std::min(27, wc.n_cells) * wc.n_atoms > (long long)NBC_CAP * wc.n_cells) {
+        static PerDevice carved;
+        carved.get(current_device(), [] {
+            cudaFuncSetAttribute(k_nbr_count_cell<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 85);
+            return 1;
+        });
+        launch_dep(k_nbr_count_cell<true>, wc.n_cells, NBC_WARPS * 32, 0, st, wc, r_list * r_list, r_sub * r_sub);
+    } else {
+        launch_dep(k_nbr_count_cell<false>, wc.n_cells, NBC_WARPS * 32, 0, st, wc, r_list * r_list, r_sub * r_sub);
+    }
     count_launch();
     // the full list's and the sub-list's row offsets in one launch
     scan_ints(wc, wc.counts, row_ptr, capacity, wc.total, wc.counts_sub, wc.counts_sub ? sub_row : nullptr,
               sub_capacity, nullptr, wc.n_atoms, st);
     if (col) {
-        launch_dep(k_nbr_fill_warp, nb, NB_WARPS * 32, 0, st, wc, r_list * r_list, row_ptr, col, x_ref, r_sub * r_sub,
+        // room for rows longer than the count keeps: those are swept and sorted again,
+        // which lives on L1 (launch.cuh; 20,000 atoms, 411 neighbours each: a build
+        // 13.7 ms early, 13.5 ordinary; rows of water early 116 us, ordinary 124)
+        launch_dep_if(capacity < 128LL * wc.n_atoms, k_nbr_fill_warp, nb, NB_WARPS * 32, 0, st, wc, r_list * r_list, row_ptr, col, x_ref, r_sub * r_sub,
                                                       wc.counts_sub ? sub_row : nullptr,
                                                       wc.counts_sub ? sub_col : nullptr);
         count_launch();
