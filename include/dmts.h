@@ -564,8 +564,7 @@ dmts_status dmts_check_bounded_wait(dmts_ctx *ctx, int limit_us, void *stream);
  * over the grid that a state's list rebuild passes between its phases (limit
  * there: 10 s): one launch of two blocks that meet at it with a limit of
  * limit_us, or, with absent = 0 or 1, of which that block never comes. The
- * other's wait then runs out (after twice limit_us where block 0 is absent)
- * and dmts_sync() returns DMTS_E_TIMEOUT once; with absent = -1 it returns
+ * other's wait then runs out and dmts_sync() returns DMTS_E_TIMEOUT once; with absent = -1 it returns
  * DMTS_OK. limit_us in [1, 1000000], else DMTS_E_INVALID. */
 dmts_status dmts_check_bounded_barrier(dmts_ctx *ctx, int limit_us, int absent, void *stream);
 

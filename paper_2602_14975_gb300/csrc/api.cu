@@ -884,7 +884,7 @@ dmts_status init_state(dmts_ctx *ctx, dmts_state *stt, float skin, cudaStream_t 
     const long long want_nc = (long long)(tot * frac * 1.6) + 16LL * N + 1024;
     if (!si->cons_col.ensure(sizeof(int) * want_cons) || !si->nc_col.ensure(sizeof(int) * want_nc) ||
         !si->scratch.slots.ensure(sizeof(int) * (size_t)N * kNbrSlots) ||
-        !ensure_zeroed(ctx, si->scratch.sync, sizeof(unsigned) * (2 + kRebuildBlocks), st))
+        !ensure_zeroed(ctx, si->scratch.sync, sizeof(unsigned) * kRebuildSyncWords, st))
         return fail(ctx, DMTS_E_OOM, "neighbour list allocation failed");
     si->cons_cap = (long long)(si->cons_col.cap / sizeof(int));
     si->nc_cap = (long long)(si->nc_col.cap / sizeof(int));

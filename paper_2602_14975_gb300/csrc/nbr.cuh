@@ -63,9 +63,9 @@ void nbr_fill(const NbrWork &w, float r_list, int *row_ptr, int *col, long long 
               float *x_ref, cudaStream_t st, float r_sub = 0.f, int *sub_row = nullptr, int *sub_col = nullptr,
               long long sub_capacity = -1);
 // The same, cells included, as one cooperative launch that does nothing while
-// *gate is 0 and clears it when done. sync: 2 + kRebuildBlocks words, zero when
+// *gate is 0 and clears it when done. sync: kRebuildSyncWords, zero when
 // allocated.
-constexpr int kRebuildBlocks = 1024;
+constexpr int kRebuildBlocks = 1024, kRebuildSyncWords = 512;
 void nbr_rebuild(const NbrWork &w, float r_list, int *row_ptr, int *col, long long capacity, float *x_ref,
                  unsigned *sync, int *gate, cudaStream_t st, float r_sub = 0.f, int *sub_row = nullptr,
                  int *sub_col = nullptr, long long sub_capacity = -1);
