@@ -51,3 +51,48 @@ def test_two_threads_with_different_species_counts(C, lmax):
         t.join()
     assert not refused, (len(refused), refused[:4])
     assert wrong == [False, False]
+
+
+def test_three_threads_rebuilding_at_once():
+    """States of three contexts stepped from three threads, on streams of
+    different priority, every inner step with a rebuild whose grid alone fills
+    the GPU: the bits of a state stepped alone."""
+    cs, ns = S.cons_spec(1, 32, 0), S.nc_spec(32, rc=3.5)
+    n = 10000
+    sy = S.water_box(n, 12.42 / 64 ** (1 / 3) * n ** (1 / 3), 1)
+    m = sy.element_masses()
+    v = S.maxwell_boltzmann(m, 300.0, 5)
+    ig = core.integrator(0.1, 5, 300.0, [20.0] * 5, skin=2e-4)
+
+    def state():
+        ctx = core.Context(cons=(cs, S.cons_weights(cs, 1)), nc=(ns, S.nc_weights(ns, 2)))
+        return ctx, core.MDState(core.DeviceSystem(sy), v, m.astype("float32"), seeds=7)
+
+    def run(ctx, st, stream, out):
+        try:
+            with torch.cuda.stream(stream):
+                for n_outer in (1, 3, 6, 1, 1):
+                    core.respa_step(ctx, st, ig, n_outer)
+                ctx.sync()
+                out.append(st.dsys.x.clone())
+                stream.synchronize()
+        except Exception as e:   # noqa: BLE001 (reported below)
+            out.append(repr(e))
+
+    alone, together = [], []
+    ctx, st = state()
+    torch.cuda.synchronize()
+    run(ctx, st, torch.cuda.Stream(), alone)
+    st.release()
+    jobs = [state() for _ in range(3)]
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=run, args=(*j, torch.cuda.Stream(priority=-k), together))
+               for k, j in enumerate(jobs)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert [o for o in alone + together if isinstance(o, str)] == []
+    assert all(torch.equal(o, alone[0]) for o in together)
+    for _, st in jobs:
+        st.release()
