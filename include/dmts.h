@@ -239,7 +239,8 @@ dmts_status nbr_build_noalloc(const dmts_system *sys, dmts_nbr *nbr, long long *
  * only). nbr must hold a list with r_list >= model rc (and >= lj_rc with
  * DMTS_WITH_PRIOR), built for the current positions. The forces are the
  * hand-written adjoint of the energy with per-layer recomputation of all
- * edge quantities; only node features are stored. Each pair's force is
+ * edge quantities; only node features are stored. Each pair's force (in the
+ * first layer each directed edge's) is
  * formed once and added to its two atoms in 32.32 fixed point, so the forces
  * do not depend on the order of the additions (the same bits alone or
  * batched); a pair term that is not finite or exceeds 2^24 in magnitude
